@@ -72,7 +72,7 @@ struct Plan {
   // device
   Item* d_items = nullptr;
   Tile* d_tiles = nullptr;
-  int32_t* d_lists = nullptr;
+  TileBox* d_boxes = nullptr;  // the tiles' box lists
   int n_tiles = 0;
   // items grouped by K (one kernel launch per group)
   struct Group {
@@ -348,7 +348,7 @@ Model* find_model(e2e_ctx* ctx, uint64_t id) {
 void free_plan(Plan& p) {
   cudaFree(p.d_items);
   cudaFree(p.d_tiles);
-  cudaFree(p.d_lists);
+  cudaFree(p.d_boxes);
   cudaFree(p.d_tile_of);
   cudaFree(p.d_grid_off);
   cudaFree(p.d_zero_tiles);
@@ -509,7 +509,12 @@ int plan_bands_and_tiles(Model* m) {
       for (int tx = it.bx0 / kTileW; tx <= (it.bx0 + it.bw - 1) / kTileW; ++tx)
         lists[tile_base[d] + ty * ntx[d] + tx].push_back((int32_t)n);
   }
-  std::vector<int32_t> flat;
+  std::vector<TileBox> flat;
+  {
+    size_t n = 0;
+    for (const auto& l : lists) n += l.size();
+    flat.reserve(n);
+  }
   P.tile_first.clear();
   for (int b = 0; b < P.n_bands; ++b) {
     P.tile_first.push_back((int)tiles.size());
@@ -518,7 +523,10 @@ int plan_bands_and_tiles(Model* m) {
         for (int tx = 0; tx < ntx[d]; ++tx) {
           const auto& l = lists[tile_base[d] + ty * ntx[d] + tx];
           Tile t{d, tx * kTileW, ty * kTileH, (int)l.size(), (int64_t)flat.size()};
-          flat.insert(flat.end(), l.begin(), l.end());
+          for (int32_t n : l) {
+            const Item& it = P.items[n];
+            flat.push_back(TileBox{(uint16_t)it.bx0, (uint16_t)it.by0, (uint16_t)it.bw, (uint16_t)it.bh, it.store_off});
+          }
           tiles.push_back(t);
         }
   }
@@ -534,7 +542,7 @@ int plan_bands_and_tiles(Model* m) {
   P.n_zero_tiles = (int)zero_tiles.size();
   int rc = upload(&P.d_items, P.items.data(), P.items.size());
   if (rc == E2E_OK) rc = upload(&P.d_tiles, tiles.data(), tiles.size());
-  if (rc == E2E_OK) rc = upload(&P.d_lists, flat.data(), flat.size());
+  if (rc == E2E_OK) rc = upload(&P.d_boxes, flat.data(), flat.size());
   if (rc == E2E_OK) rc = upload(&P.d_tile_of, tile_of.data(), tile_of.size());
   if (rc == E2E_OK) rc = upload(&P.d_grid_off, grid_off.data(), grid_off.size());
   if (rc == E2E_OK) rc = upload(&P.d_zero_tiles, zero_tiles.data(), zero_tiles.size());
@@ -915,7 +923,7 @@ int render_impl(e2e_ctx* ctx, Model* m, int n_spec, const uint64_t* spec_ids, in
     int* count = nullptr;
     E2E_CK(sc.get((void**)&count, (size_t)P.n_tiles * sizeof(int)));
     if (count) E2E_CK(cudaMemsetAsync(count, 0, (size_t)P.n_tiles * sizeof(int), st));
-    const MergeArgs mg{P.d_items, P.d_tiles, P.d_lists, P.d_tile_of, P.d_grid_off, m->d_dims, count, d_dst, d_pitch,
+    const MergeArgs mg{P.d_tiles, P.d_boxes, P.d_tile_of, P.d_grid_off, m->d_dims, count, d_dst, d_pitch,
                        dtype == E2E_F32 ? 0 : 1, nullptr, 0};
     bool zeros = false;  // the zero tiles ride as extra CTAs at the end of the first non-empty launch
     for (auto& g : P.groups) {
@@ -930,7 +938,7 @@ int render_impl(e2e_ctx* ctx, Model* m, int n_spec, const uint64_t* spec_ids, in
     }
     if (!zeros) {  // no item at all: every tile is a zero tile
       KernelTimer kt(ctx, st, "merge_zero");
-      E2E_CK(launch_merge(P.d_zero_tiles, P.n_zero_tiles, P.d_lists, P.d_items, store, d_dst, dtype, d_pitch,
+      E2E_CK(launch_merge(P.d_zero_tiles, P.n_zero_tiles, P.d_boxes, store, d_dst, dtype, d_pitch,
                           m->d_dims, st));
     }
   } else {
@@ -939,7 +947,7 @@ int render_impl(e2e_ctx* ctx, Model* m, int n_spec, const uint64_t* spec_ids, in
       E2E_CK(launch_items(ctx, m, g.K, g.first, g.count, d_table, store, st));
     }
     KernelTimer kt(ctx, st, "merge");
-    E2E_CK(launch_merge(P.d_tiles, P.n_tiles, P.d_lists, P.d_items, store, d_dst, dtype, d_pitch, m->d_dims, st));
+    E2E_CK(launch_merge(P.d_tiles, P.n_tiles, P.d_boxes, store, d_dst, dtype, d_pitch, m->d_dims, st));
   }
   if (ctx->d_err) {  // debug checks: wait for the render and report unplanned deposits
     int n_bad = 0;
@@ -1040,7 +1048,7 @@ int render_host_banded(e2e_ctx* ctx, Model* m, int n_spec, const uint64_t* spec_
     }
     E2E_CK(cudaEventRecord(ev[1 + b], r));
     E2E_CK(cudaStreamWaitEvent(M, ev[1 + b], 0));  // bands < b: waited for by earlier merges
-    E2E_CK(launch_merge(P.d_tiles + P.tile_first[b], P.tile_first[b + 1] - P.tile_first[b], P.d_lists, P.d_items,
+    E2E_CK(launch_merge(P.d_tiles + P.tile_first[b], P.tile_first[b + 1] - P.tile_first[b], P.d_boxes,
                         store, d_dst, dtype, d_pitch, m->d_dims, M));
     E2E_CK(cudaEventRecord(ev[1 + kBands + b], M));
     E2E_CK(cudaStreamWaitEvent(C, ev[1 + kBands + b], 0));
@@ -1723,7 +1731,7 @@ int e2e_render_static(e2e_ctx* ctx, uint64_t model_id, int32_t n_spec, const uin
   }
   {
     KernelTimer kt(ctx, st, "merge");
-    E2E_CK(launch_merge(P.d_tiles, P.n_tiles, P.d_lists, P.d_items, store, d_dst, dtype, d_pitch, m->d_dims, st));
+    E2E_CK(launch_merge(P.d_tiles, P.n_tiles, P.d_boxes, store, d_dst, dtype, d_pitch, m->d_dims, st));
   }
   if (ctx->d_err) {  // debug checks: wait for the render and report unplanned deposits
     int n_bad = 0;

@@ -64,7 +64,14 @@ struct TableSlice {
 // row starts on a 128-byte line and a warp's 32 consecutive reads touch 4 sectors, not 5.
 __host__ __device__ constexpr int table_row32(int K) { return (K * K + 31) / 32 * 32; }
 
-// Output tile of the merge: tile (tx, ty) of detector det lists items[list_off .. list_off+n).
+// An entry of a merge tile's list: an item's box (on the detector, so below 2^16) and its offset
+// in the box store.
+struct __align__(16) TileBox {
+  uint16_t bx0, by0, bw, bh;
+  int64_t off;
+};
+
+// Output tile of the merge: tile (tx, ty) of detector det lists boxes[list_off .. list_off+n).
 struct Tile {
   int32_t det, x0, y0, n;
   int64_t list_off;

@@ -15,9 +15,8 @@ constexpr int kStaticSmemReserve = 1024;  // static shared memory of the render 
 // The fused tile merge of the separable render kernel (merge_tile.cuh): per-tile item counts,
 // the plan's tiles and lists, and the frames.  count == nullptr: no fused merge.
 struct MergeArgs {
-  const Item* items;        // the plan's items (the tile lists hold indices into this array)
   const Tile* tiles;
-  const int32_t* lists;     // CSR item lists of the tiles (item order)
+  const TileBox* boxes;     // the tiles' box lists (item order)
   const int32_t* tile_of;   // tile index of (detector, tile row, tile column)
   const int32_t* grid_off;  // per detector: its first entry in tile_of
   const int* dims;          // per detector: (H, W)
@@ -45,7 +44,7 @@ cudaError_t launch_render_mixed(int K, int DX, int DY, const DevSlice* slices, c
                                 const double* u_all, const Item* items, int n_items, float2* store, int B, int JB,
                                 int nk_max, int max_deg, int far_tails, size_t smem, cudaStream_t st,
                                 int* err = nullptr, const MergeArgs* mg = nullptr);
-cudaError_t launch_merge(const Tile* tiles, int n_tiles, const int32_t* lists, const Item* items, const float2* store,
+cudaError_t launch_merge(const Tile* tiles, int n_tiles, const TileBox* boxes, const float2* store,
                          void* const* dst, int dtype, const int64_t* pitch, const int* dims, cudaStream_t st);
 
 size_t ellip_smem_bytes(int area, int nk_max, int nd, int k_min);

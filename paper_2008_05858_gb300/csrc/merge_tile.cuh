@@ -16,52 +16,96 @@
 
 namespace e2e {
 
-// Merge tile t with NT threads (thread index tid); box reads bypass L1 when CG (the boxes were
-// written by other CTAs during this launch).
-template <int NT, bool CG, typename T>
-__device__ __forceinline__ void merge_tile(const Tile& t, const int32_t* __restrict__ lists,
-                                           const Item* __restrict__ items, const float2* store, T* frame, int64_t P,
-                                           int H, int W, int tid) {
-  constexpr int kRows = kTileW * kTileH / NT;  // pixels per thread
-  constexpr int kStep = NT / kTileW;
-  const int tx = tid & (kTileW - 1), ty0 = tid / kTileW;
-  const int x = t.x0 + tx;
-  if (t.n == 0) {
-    if (x < W) {
+// A warp merges 32 neighbouring columns x kMergeRows rows at a time.
+constexpr int kMergeRows = 8;
+constexpr int kMergeBlocks = (kTileW / 32) * (kTileH / kMergeRows);  // such sub-blocks of a tile
+// Boxes whose pixels of a sub-block are loaded together: the latency of a load from L2 is paid
+// once per kMergeDepth boxes; their pixels are still added one box after the other.
+constexpr int kMergeDepth = 2;
+
+// Entry `lane` of tile t's list (zeros beyond its end).
+__device__ __forceinline__ TileBox tile_entry(const Tile& t, const TileBox* __restrict__ boxes, int lane) {
+  return lane < t.n ? boxes[t.list_off + lane] : TileBox{};
+}
+
+// Merge sub-block blk of tile t, by one warp; box reads bypass L1 when CG (the boxes were written
+// by other CTAs during this launch).
+//
+// Of the boxes in a tile's list (6 on the full-detector frame, 24 on a finely sampled 1024 x 256
+// tile) only two to four reach a given sub-block.  Following the list item by item (its index, the
+// item, then its pixels) cost three loads from L2 per item, one after the other.  Here the lanes
+// load 32 list entries at once, which hold the boxes themselves, each lane tests its box against
+// the sub-block, and the warp walks the set bits of the ballot.  The boxes are added in list order.
+// `first` is this lane's entry of the list's first 32 (any value beyond the list's end).
+template <bool CG, typename T>
+__device__ __forceinline__ void merge_block(const Tile& t, const TileBox& first, const TileBox* __restrict__ boxes,
+                                            const float2* store, T* frame, int64_t P, int H, int W, int blk,
+                                            int lane) {
+  const int x0 = t.x0 + (blk % (kTileW / 32)) * 32, y0 = t.y0 + (blk / (kTileW / 32)) * kMergeRows;
+  if (x0 >= W || y0 >= H) return;
+  float sum[kMergeRows], comp[kMergeRows];
 #pragma unroll
-      for (int q = 0; q < kRows; ++q) {
-        const int y = t.y0 + ty0 + q * kStep;
-        if (y < H) frame[(int64_t)y * P + x] = (T)0;
+  for (int q = 0; q < kMergeRows; ++q) sum[q] = comp[q] = 0.f;
+  for (int n0 = 0; n0 < t.n; n0 += 32) {
+    TileBox b = first;
+    bool hit = false;
+    if (n0 + lane < t.n) {
+      if (n0 > 0) b = boxes[t.list_off + n0 + lane];
+      hit = b.bx0 < x0 + 32 && b.bx0 + b.bw > x0 && b.by0 < y0 + kMergeRows && b.by0 + b.bh > y0;
+    }
+    unsigned m = __ballot_sync(0xffffffffu, hit);
+    const int xy = b.bx0 | (b.by0 << 16), wh = b.bw | (b.bh << 16);
+    while (m) {
+      float2 v[kMergeDepth][kMergeRows];
+      const int nd = min(kMergeDepth, __popc(m));
+#pragma unroll
+      for (int d = 0; d < kMergeDepth; ++d) {
+        if (d < nd) {  // uniform over the warp
+          const int i = __ffs(m) - 1;
+          m &= m - 1;
+          const unsigned ixy = __shfl_sync(0xffffffffu, xy, i), iwh = __shfl_sync(0xffffffffu, wh, i);
+          const int64_t off = __shfl_sync(0xffffffffu, b.off, i);
+          const int bw = iwh & 0xffff, bh = iwh >> 16;
+          const int gx = x0 + lane - (int)(ixy & 0xffff), gy = y0 - (int)(ixy >> 16);
+          const float2* p = store + off + (int64_t)gy * bw + gx;
+          const bool inx = (unsigned)gx < (unsigned)bw;
+#pragma unroll
+          for (int q = 0; q < kMergeRows; ++q) {
+            const bool in = inx && (unsigned)(gy + q) < (unsigned)bh;
+            v[d][q] = in ? (CG ? __ldcg(p + q * bw) : p[q * bw]) : make_float2(0.f, 0.f);
+          }
+        }
+      }
+#pragma unroll
+      for (int d = 0; d < kMergeDepth; ++d) {
+        if (d < nd) {
+#pragma unroll
+          for (int q = 0; q < kMergeRows; ++q) {
+            float s, e;
+            two_sum(sum[q], v[d][q].x, s, e);
+            sum[q] = s;
+            comp[q] += e + v[d][q].y;
+          }
+        }
       }
     }
-    return;
   }
-  float sum[kRows], comp[kRows];
-#pragma unroll
-  for (int q = 0; q < kRows; ++q) sum[q] = comp[q] = 0.f;
-  for (int n = 0; n < t.n; ++n) {
-    const Item it = items[lists[t.list_off + n]];
-    const int gx = x - it.bx0;
-    if (gx < 0 || gx >= it.bw) continue;
-    const float2* box = store + it.store_off;
-#pragma unroll
-    for (int q = 0; q < kRows; ++q) {
-      const int gy = t.y0 + ty0 + q * kStep - it.by0;
-      if (gy >= 0 && gy < it.bh) {
-        const float2 v = CG ? __ldcg(box + (int64_t)gy * it.bw + gx) : box[(int64_t)gy * it.bw + gx];
-        float s, e;
-        two_sum(sum[q], v.x, s, e);
-        sum[q] = s;
-        comp[q] += e + v.y;
-      }
-    }
-  }
+  const int x = x0 + lane;
   if (x >= W) return;
+  T* out = frame + (int64_t)y0 * P + x;
 #pragma unroll
-  for (int q = 0; q < kRows; ++q) {
-    const int y = t.y0 + ty0 + q * kStep;
-    if (y < H) frame[(int64_t)y * P + x] = sizeof(T) == 8 ? (T)((double)sum[q] + (double)comp[q]) : (T)(sum[q] + comp[q]);
-  }
+  for (int q = 0; q < kMergeRows; ++q)
+    if (y0 + q < H) out[q * P] = sizeof(T) == 8 ? (T)((double)sum[q] + (double)comp[q]) : (T)(sum[q] + comp[q]);
+}
+
+// Merge tile t with the NT threads (whole warps) of a CTA.
+template <int NT, bool CG, typename T>
+__device__ __forceinline__ void merge_tile(const Tile& t, const TileBox* __restrict__ boxes, const float2* store,
+                                           T* frame, int64_t P, int H, int W, int tid) {
+  const int lane = tid & 31;
+  const TileBox first = tile_entry(t, boxes, lane);
+  for (int blk = tid >> 5; blk < kMergeBlocks; blk += NT / 32)
+    merge_block<CG, T>(t, first, boxes, store, frame, P, H, W, blk, lane);
 }
 
 // End of a render CTA of NT threads that has written item `it`'s box (every thread's stores
@@ -70,7 +114,6 @@ template <int NT>
 __device__ void fused_merge_epilogue(const MergeArgs& g, const float2* store, const Item& it, int det) {
   __shared__ int s_tiles[NT];
   __shared__ int s_n;
-  const Item* __restrict__ items = g.items;
   __threadfence();  // this thread's box stores are visible device-wide
   __syncthreads();  // ... and every thread's, before any count of this CTA
   const int W = g.dims[2 * det + 1], H = g.dims[2 * det];
@@ -98,10 +141,10 @@ __device__ void fused_merge_epilogue(const MergeArgs& g, const float2* store, co
       for (int k = 0; k < m; ++k) {
         const Tile t = g.tiles[s_tiles[k]];
         if (g.dtype == 0)
-          merge_tile<NT, true, float>(t, g.lists, items, store, static_cast<float*>(g.dst[t.det]), g.pitch[t.det], H, W,
+          merge_tile<NT, true, float>(t, g.boxes, store, static_cast<float*>(g.dst[t.det]), g.pitch[t.det], H, W,
                                       threadIdx.x);
         else
-          merge_tile<NT, true, double>(t, g.lists, items, store, static_cast<double*>(g.dst[t.det]), g.pitch[t.det], H,
+          merge_tile<NT, true, double>(t, g.boxes, store, static_cast<double*>(g.dst[t.det]), g.pitch[t.det], H,
                                        W, threadIdx.x);
       }
     }

@@ -106,13 +106,19 @@ size_t mixed_smem_bytes(int area, int JB, int nk_max, int B, int nd) {
 
 // ------------------------------------------------------------------------------ merge
 
-// One CTA of 256 threads per output tile (merge_tile.cuh).  Tiles that no item touches are zeros.
+// One CTA of 256 threads per output tile, a warp per sub-block (merge_tile.cuh); tiles that no
+// item touches are zeros.  What bounds it is the chain of loads of each sub-block (the tile, its
+// boxes, their pixels) and the instructions around them: 296 us for the full-detector frame's 820
+// MB of boxes and frame, against 467 us with the boxes looked up through the item list.  Four rows
+// a warp (512 threads, 40 registers) took 312 us, a persistent grid with the next tile's boxes
+// prefetched 415 us (64 registers, spilled).
 template <typename T>
-__global__ void __launch_bounds__(256) k_merge(const Tile* __restrict__ tiles, const int32_t* __restrict__ lists,
-                                               const Item* __restrict__ items, const float2* __restrict__ store,
-                                               T* const* dst, const int64_t* __restrict__ pitch, const int* __restrict__ dims) {
+__global__ void __launch_bounds__(256) k_merge(const Tile* __restrict__ tiles, const TileBox* __restrict__ boxes,
+                                               const float2* __restrict__ store, T* const* dst,
+                                               const int64_t* __restrict__ pitch, const int* __restrict__ dims) {
+  static_assert(kMergeBlocks == 8, "one warp of the CTA per sub-block");
   const Tile t = tiles[blockIdx.x];
-  merge_tile<256, false, T>(t, lists, items, store, dst[t.det], pitch[t.det], dims[2 * t.det], dims[2 * t.det + 1],
+  merge_tile<256, false, T>(t, boxes, store, dst[t.det], pitch[t.det], dims[2 * t.det], dims[2 * t.det + 1],
                             threadIdx.x);
 }
 
@@ -154,13 +160,13 @@ cudaError_t launch_render_mixed(int K, int DX, int DY, const DevSlice* slices, c
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_merge(const Tile* tiles, int n_tiles, const int32_t* lists, const Item* items, const float2* store,
+cudaError_t launch_merge(const Tile* tiles, int n_tiles, const TileBox* boxes, const float2* store,
                          void* const* dst, int dtype, const int64_t* pitch, const int* dims, cudaStream_t st) {
   if (n_tiles == 0) return cudaSuccess;
   if (dtype == 0)
-    k_merge<float><<<n_tiles, 256, 0, st>>>(tiles, lists, items, store, (float* const*)dst, pitch, dims);
+    k_merge<float><<<n_tiles, 256, 0, st>>>(tiles, boxes, store, (float* const*)dst, pitch, dims);
   else
-    k_merge<double><<<n_tiles, 256, 0, st>>>(tiles, lists, items, store, (double* const*)dst, pitch, dims);
+    k_merge<double><<<n_tiles, 256, 0, st>>>(tiles, boxes, store, (double* const*)dst, pitch, dims);
   return cudaGetLastError();
 }
 

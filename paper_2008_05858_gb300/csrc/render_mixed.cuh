@@ -99,10 +99,10 @@ __global__ void __launch_bounds__(kThreads, mixed_min_blocks<K, DX, DY>()) k_ren
     const Tile t = mg.zero_tiles[blockIdx.x - (gridDim.x - mg.n_zero)];
     const int th = mg.dims[2 * t.det], tw = mg.dims[2 * t.det + 1];
     if (mg.dtype == 0)
-      merge_tile<kThreads, false, float>(t, mg.lists, mg.items, a.store, reinterpret_cast<float* const*>(mg.dst)[t.det],
+      merge_tile<kThreads, false, float>(t, mg.boxes, a.store, reinterpret_cast<float* const*>(mg.dst)[t.det],
                                          mg.pitch[t.det], th, tw, threadIdx.x);
     else
-      merge_tile<kThreads, false, double>(t, mg.lists, mg.items, a.store, reinterpret_cast<double* const*>(mg.dst)[t.det],
+      merge_tile<kThreads, false, double>(t, mg.boxes, a.store, reinterpret_cast<double* const*>(mg.dst)[t.det],
                                           mg.pitch[t.det], th, tw, threadIdx.x);
     return;
   }
