@@ -91,10 +91,23 @@ __global__ void k_plan(const DevSlice* __restrict__ slices, int n_slices, const 
       atomicMin(&bb->z, ymn - h);
       atomicMax(&bb->w, ymx + h);
     }
+    // A slice's ten spans take the maxima of all its threads: 32 lanes of one slice are reduced
+    // first, and a maximum already reached is only read (every thread adding to those few
+    // addresses was nine tenths of this kernel: 0.33 ms of a fitting iteration).
+    const unsigned active = __activemask();
+    const bool one = __all_sync(active, lo == __shfl_sync(active, lo, __ffs(active) - 1));
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
-      atomicMax(&spans[(lo * 5 + q) * 2 + 0], spx[q]);
-      atomicMax(&spans[(lo * 5 + q) * 2 + 1], spy[q]);
+      int* sp = spans + (lo * 5 + q) * 2;
+      int mx = spx[q], my = spy[q];
+      if (one) {
+        mx = __reduce_max_sync(active, mx);
+        my = __reduce_max_sync(active, my);
+      }
+      if (!one || (threadIdx.x & 31) == __ffs(active) - 1) {
+        if (mx > __ldcg(sp)) atomicMax(sp, mx);
+        if (my > __ldcg(sp + 1)) atomicMax(sp + 1, my);
+      }
     }
   }
 }
