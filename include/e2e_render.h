@@ -53,8 +53,10 @@ extern "C" {
 /* ------------------------------------------------------------------ enums */
 enum { E2E_PSF_SEPARABLE = 0, E2E_PSF_ELLIPTICAL = 1, E2E_PSF_TABLE = 2 };
 /* E2E_PREC_MIXED: the mapping's per-sample coefficients in FP64, its polynomial in the slit
- *                 coordinate in double-float FP32 (within ~1e-10 px of FP64); FP32 PSF stamps
- *                 from double-float edge arguments; FP32 sums
+ *                 coordinate in double-float FP32 (within ~1e-10 px of FP64; the windows are
+ *                 those of that mapping, the offset in the pixel may be rounded to ~1e-7 px);
+ *                 FP32 PSF stamps, from polynomials in that offset where a separable model's
+ *                 widths stay >= 1 px, else from double-float edge arguments; FP32 sums
  *                 over runs of <= 16 stamps in registers; each item's box summed exactly in
  *                 52-bit fixed point (shared-memory integer atomics) and stored as an FP32
  *                 (hi, lo) pair; boxes merged into the frame with TwoSum compensation (the
@@ -171,8 +173,10 @@ const char* e2e_last_error(void);
  * device and plans the tiled render (synchronous; uses the context's device).  Resident per
  * model: the slices, the plan (items, merge tiles and their lists), and per wavelength sample
  * of every slice (degree + 3) x 16 bytes of precomputed mapping coefficients and PSF constants
- * (261 MB for a 9216^2 frame of 340 slices x 6000 samples at degree 5); the tabulated PSF adds
- * its coefficient tables.
+ * (261 MB for a 9216^2 frame of 340 slices x 6000 samples at degree 5); a separable model whose
+ * widths stay >= 1 px and windows K >= 3 adds its pixel-integral polynomials, 512 bytes per sample
+ * at K = 11 (1.04 GB for that frame; left out where the device has no room for them); the
+ * tabulated PSF adds its coefficient tables.
  * Errors: E2E_EINVAL, E2E_ENOMEM, E2E_ECUDA. */
 int e2e_load_model(e2e_ctx* ctx, const e2e_model_desc* desc, uint64_t* model_id);
 int e2e_unload_model(e2e_ctx* ctx, uint64_t model_id);

@@ -24,6 +24,7 @@
 #include "../../include/e2e_render.h"
 #include "e2e_device.cuh"
 #include "e2e_kernels.h"
+#include "poly_tables.cuh"
 #include "tail_coeffs.h"
 
 using namespace e2e;
@@ -65,6 +66,8 @@ struct SliceHost {
 struct Plan {
   bool ok = false;
   int B = 1, DX = 0, DY = 0, JB = 1, NB = 8, max_area = 0, max_deg = 0, nk_max = 1;
+  int B_adj = 1;      // run length of the adjoint (its FP32 sums run over one run)
+  int poly = 0;       // separable kernel: polynomial pixel integrals (every sample's table is built)
   int far_tails = 0;  // separable kernel: every tail edge's argument within the cheaper rational's fit
   std::vector<Item> items;  // host copy
   int64_t store_elems = 0;
@@ -95,6 +98,7 @@ struct Plan {
   int n_zero_tiles = 0;
 };
 
+constexpr int kPolyWave = 152 * 4;  // CTAs of the polynomial kernel the GPU holds at once
 constexpr int kBands = 16;  // y-bands of a frame rendered into host memory
 
 struct Model {
@@ -133,6 +137,7 @@ struct Model {
   int parent_coef_total = 0;
   int* d_fold = nullptr;  // first_sub | sub coef_off | parent coef_off | parent nc (adjoint folding)
   float4* d_stab = nullptr;  // per-sample tables of every slice (DevSlice::samples)
+  bool has_poly = false;     // ... followed by the polynomial pixel integrals (DevSlice::poly)
 };
 
 struct Spectrum {
@@ -400,6 +405,15 @@ double variant_cost(int K, int DX, int DY, int B) {
   return c;
 }
 
+// The same for the polynomial kernel, in lane operations per stamp: each lane of the quad
+// evaluates its half of one axis (~45) and adds its quadrant of the tile (half an operation per
+// pixel, packed, and the loads of its rows and columns); per run the quadrant is cleared and
+// flushed (~8 operations per pixel).
+double poly_variant_cost(int K, int DX, int DY, int B) {
+  const double nx = (K + DX + 1) / 2, ny = (K + DY + 1) / 2;
+  return 4.0 * (45.0 + 0.5 * nx * ny + nx + ny + 8.0 * nx * ny / B);
+}
+
 // Phase-cell tables of a tabulated-PSF model, built on the device at load time.
 int build_psf_tables(Model* m) {
   NvtxRange nvtx_("e2e psf tables");
@@ -563,11 +577,39 @@ int build_sample_tables(Model* m) {
     total += (int64_t)m->dev[i].n_lambda * (m->dev[i].degree + 3);
     max_lambda = std::max(max_lambda, m->dev[i].n_lambda);
   }
-  if (!m->d_stab) E2E_CK(cudaMalloc((void**)&m->d_stab, (size_t)total * sizeof(float4)));
+  // polynomial pixel integrals, where the model's narrowest PSF allows them, in the same
+  // allocation; a device without room for them renders from the edge tails instead
+  std::vector<int64_t> poff(ns);
+  int64_t ptotal = 0;
+  bool can = m->psf == E2E_PSF_SEPARABLE, poly = true;
+  for (int i = 0; i < ns && can; ++i) {
+    const auto& s = m->slices[i].d;
+    can = poly_variant_supported(s.K);
+    poly = poly && std::min(quad_min(s.sigma_x), quad_min(s.sigma_y)) >= kPolyMinSigma;
+    poff[i] = total + ptotal;
+    ptotal += (int64_t)s.n_lambda * poly_row_f4(s.K);
+  }
+  poly = poly && can;
+  if (poly && !m->has_poly) {  // an update widened the PSF: make room for the polynomials
+    cudaFree(m->d_stab);
+    m->d_stab = nullptr;
+  }
+  if (!m->d_stab) {
+    if (poly && cudaMalloc((void**)&m->d_stab, (size_t)(total + ptotal) * sizeof(float4)) == cudaSuccess) {
+      m->has_poly = true;
+    } else {
+      cudaGetLastError();
+      E2E_CK(cudaMalloc((void**)&m->d_stab, (size_t)total * sizeof(float4)));
+    }
+  }
+  poly = poly && m->has_poly;
   for (int i = 0; i < ns; ++i) m->dev[i].samples = m->d_stab + off[i];
+  m->plan.poly = poly ? 1 : 0;
+  for (int i = 0; i < ns; ++i) m->dev[i].poly = poly ? m->d_stab + poff[i] : nullptr;
   E2E_CK(cudaMemcpy(m->d_slices, m->dev.data(), ns * sizeof(DevSlice), cudaMemcpyHostToDevice));
   const int psf = m->psf == E2E_PSF_ELLIPTICAL ? 1 : m->psf == E2E_PSF_TABLE ? 2 : 0;
   E2E_CK(launch_sample_tables(m->d_slices, ns, max_lambda, psf, m->d_ts, m->d_field, 0));
+  if (poly) E2E_CK(launch_poly_tables(m->d_slices, ns, max_lambda, 0));
   E2E_CK(cudaDeviceSynchronize());
   return E2E_OK;
 }
@@ -615,7 +657,7 @@ int plan_model(Model* m) {
   // elliptical kernel has no run tiles: one item per (32-sample, 16-point) block.
   int K = 0;
   for (auto& s : m->slices) K = std::max(K, s.d.K);
-  double best = 1e300;
+  double best = 1e300, best_tail = 1e300;
   int bB = 1, bDX = 0, bDY = 0;
   const int variants[5][2] = {{0, 0}, {1, 1}, {1, 2}, {1, 3}, {2, 2}};
   for (int q = 0; q <= 4 && !ellip; ++q) {  // B = 1..16
@@ -629,7 +671,12 @@ int plan_model(Model* m) {
       bool ok = true;
       for (int k : m->Ks) ok = ok && mixed_variant_supported(k, v[0], v[1]);
       if (!ok || sx > v[0] || sy > v[1]) continue;
-      const double c = variant_cost(K, v[0], v[1], B);
+      const double ct = variant_cost(K, v[0], v[1], B);
+      if (ct < best_tail) {
+        best_tail = ct;
+        P.B_adj = B;
+      }
+      const double c = P.poly ? poly_variant_cost(K, v[0], v[1], B) : ct;
       if (c < best) {
         best = c;
         bB = B;
@@ -719,8 +766,12 @@ int plan_model(Model* m) {
     }
     P.smem = m->psf == E2E_PSF_TABLE ? table_smem_bytes(P.max_area, P.nk_max, P.max_deg + 1)
              : ellip ? ellip_smem_bytes(P.max_area, P.nk_max, P.max_deg + 1, m->Ks.empty() ? 15 : m->Ks.front())
+             : P.poly ? poly_smem_bytes(P.max_area, P.JB, P.nk_max, P.max_deg + 1)
                      : mixed_smem_bytes(P.max_area, P.JB, P.nk_max, P.B, P.max_deg + 1);
-    if ((int)P.smem + kStaticSmemReserve <= optin) break;
+    // the polynomial kernel's warps take eight samples each through the whole slit: a grid that
+    // would not fill the GPU gets items of one 32-sample block (a sample octet per warp)
+    const bool thin = P.poly && jb_cap > 1 && P.JB > 1 && (int)P.items.size() < kPolyWave;
+    if ((int)P.smem + kStaticSmemReserve <= optin && !thin) break;
     if (jb_cap == 1)
       return fail(E2E_EINVAL, "trace footprint of a work item exceeds on-chip memory (area " +
                                   std::to_string(P.max_area) + " px)");
@@ -833,6 +884,9 @@ cudaError_t launch_items(e2e_ctx* ctx, Model* m, int K, int first, int count, co
   if (m->psf == E2E_PSF_ELLIPTICAL)
     return launch_render_ellip(K, m->d_slices, d_table, m->d_u, P.d_items + first, count, store, P.nk_max,
                                P.max_deg, P.smem, st, ctx->d_err);
+  if (P.poly)
+    return launch_render_poly(K, P.DX, P.DY, m->d_slices, d_table, m->d_u, P.d_items + first, count, store, P.B, P.JB,
+                              P.nk_max, P.max_deg, P.smem, st, ctx->d_err);
   return launch_render_mixed(K, P.DX, P.DY, m->d_slices, d_table, m->d_u, P.d_items + first, count, store, P.B,
                              P.JB, P.nk_max, P.max_deg, P.far_tails, P.smem, st, ctx->d_err, mg);
 }
@@ -917,8 +971,8 @@ int render_impl(e2e_ctx* ctx, Model* m, int n_spec, const uint64_t* spec_ids, in
   float2* store = nullptr;
   E2E_CK(sc.get((void**)&store, (size_t)P.store_elems * sizeof(float2)));
   if (ctx->d_err) E2E_CK(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), st));
-  if (!tab && !ellip) {
-    // separable PSF: the render CTA that finishes a tile's last item merges the tile; the
+  if (!tab && !ellip && !P.poly) {
+    // edge-tail kernel: the render CTA that finishes a tile's last item merges the tile; the
     // tiles no item overlaps are written as zeros first
     int* count = nullptr;
     E2E_CK(sc.get((void**)&count, (size_t)P.n_tiles * sizeof(int)));
@@ -943,7 +997,7 @@ int render_impl(e2e_ctx* ctx, Model* m, int n_spec, const uint64_t* spec_ids, in
     }
   } else {
     for (auto& g : P.groups) {
-      KernelTimer kt(ctx, st, tab ? "render_table" : "render_ellip");
+      KernelTimer kt(ctx, st, tab ? "render_table" : ellip ? "render_ellip" : "render_mixed");
       E2E_CK(launch_items(ctx, m, g.K, g.first, g.count, d_table, store, st));
     }
     KernelTimer kt(ctx, st, "merge");
@@ -1726,8 +1780,7 @@ int e2e_render_static(e2e_ctx* ctx, uint64_t model_id, int32_t n_spec, const uin
   if (ctx->d_err) E2E_CK(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), st));
   for (auto& grp : P.groups) {
     KernelTimer kt(ctx, st, "render_mixed");
-    E2E_CK(launch_render_mixed(grp.K, P.DX, P.DY, m->d_slices, d_table, m->d_u, P.d_items + grp.first, grp.count,
-                               store, P.B, P.JB, P.nk_max, P.max_deg, P.far_tails, P.smem, st, ctx->d_err));
+    E2E_CK(launch_items(ctx, m, grp.K, grp.first, grp.count, d_table, store, st));
   }
   {
     KernelTimer kt(ctx, st, "merge");
@@ -1801,12 +1854,12 @@ int e2e_render_adjoint(e2e_ctx* ctx, uint64_t model_id, int32_t n_spec, const ui
   for (const Item& it : P.items) nj_max = std::max(nj_max, it.nj);
   const size_t smem = adjoint_smem_bytes(P.max_area, P.max_deg, P.nk_max, nj_max);
   int max_tasks = 1;  // warp tasks of the largest item: 32-sample blocks x runs
-  for (const Item& it : P.items) max_tasks = std::max(max_tasks, ((it.nj + 31) / 32) * ((it.nk + P.B - 1) / P.B));
+  for (const Item& it : P.items) max_tasks = std::max(max_tasks, ((it.nj + 31) / 32) * ((it.nk + P.B_adj - 1) / P.B_adj));
   const int parts = adjoint_parts(max_tasks);
   for (auto& grp : P.groups) {
     KernelTimer kt(ctx, st, "adjoint");
     E2E_CK(launch_adjoint(grp.K, m->d_slices, d_table, m->d_u, P.d_items + grp.first, grp.count, d_dldi, d_pitch,
-                          dtype == E2E_F32 ? 0 : 1, P.B, P.nk_max, parts, g_cx, g_cy, g_sx, g_sy, smem, st,
+                          dtype == E2E_F32 ? 0 : 1, P.B_adj, P.nk_max, parts, g_cx, g_cy, g_sx, g_sy, smem, st,
                           reinterpret_cast<const int2*>(frozen_windows)));
   }
   if (m->expanded)

@@ -32,6 +32,9 @@ struct DevSlice {
   // degree + 3 float4 at samples + j (degree + 3): the s-polynomial's coefficients P_b(lt_j)
   // as split_xy pairs (b = 0..degree), then two float4 of PSF constants (see sample_tables.cu)
   const float4* samples;
+  // polynomial pixel integrals (poly_tables.cuh), or null: for wavelength sample j, the
+  // 4 poly_role_f4(K) float4 at poly + j 4 poly_role_f4(K), one block per role 2 half + axis
+  const float4* poly;
 };
 
 // A mixed-path work item: a block of wavelength samples x a block of slit points of one

@@ -44,6 +44,14 @@ cudaError_t launch_render_mixed(int K, int DX, int DY, const DevSlice* slices, c
                                 const double* u_all, const Item* items, int n_items, float2* store, int B, int JB,
                                 int nk_max, int max_deg, int far_tails, size_t smem, cudaStream_t st,
                                 int* err = nullptr, const MergeArgs* mg = nullptr);
+// The separable render on polynomial pixel integrals (render_poly.cuh; DevSlice::poly set).
+bool poly_variant_supported(int K);
+size_t poly_smem_bytes(int area, int JB, int nk_max, int nd);
+int poly_row_f4(int K);  // float4s of one sample's polynomial table
+cudaError_t launch_poly_tables(const DevSlice* slices, int n_slices, int max_lambda, cudaStream_t st);
+cudaError_t launch_render_poly(int K, int DX, int DY, const DevSlice* slices, const double* const* flux_tab,
+                               const double* u_all, const Item* items, int n_items, float2* store, int B, int JB,
+                               int nk_max, int max_deg, size_t smem, cudaStream_t st, int* err = nullptr);
 cudaError_t launch_merge(const Tile* tiles, int n_tiles, const TileBox* boxes, const float2* store,
                          void* const* dst, int dtype, const int64_t* pitch, const int* dims, cudaStream_t st);
 

@@ -60,6 +60,11 @@ __device__ __forceinline__ float2 fixed_to_pair(int hi, unsigned lo, float scale
   return make_float2(s * scale, e * scale);
 }
 
+// The same for a signed low word: its sign moved into the high word.
+__device__ __forceinline__ float2 fixed_to_pair_s(int hi, int lo, float scale) {
+  return fixed_to_pair(hi + (lo >> 22), (unsigned)lo & 0x3FFFFFu, scale);
+}
+
 // Fixed-point deposit of val into a box pixel: the value scaled by 2^P is cut into a high
 // word (multiples of 2^22, signed) and a low word (< 2^22, unsigned), both added with
 // integer atomics, so the sums are exact and independent of the order of the deposits.
@@ -68,6 +73,14 @@ __device__ __forceinline__ void box_deposit(int* hi, unsigned* lo, float val, fl
   const float lf = fmaf(-hf, 4194304.f, val * sc);
   atomicAdd(hi, __float2int_rz(hf));
   atomicAdd(lo, __float2uint_rn(lf));
+}
+
+// box_deposit with both words rounded to nearest, the low word signed.
+__device__ __forceinline__ void box_deposit_s(int* hi, int* lo, float val, float sc, float sc_hi) {
+  const float hf = rintf(val * sc_hi);
+  const float lf = fmaf(-hf, 4194304.f, val * sc);
+  atomicAdd(hi, __float2int_rz(hf));
+  atomicAdd(lo, __float2int_rn(lf));
 }
 
 // ---- the stamp mapping of the mixed-precision kernels and their planner, in double-float
@@ -249,6 +262,15 @@ __device__ __forceinline__ void fixed_split2(float2 val, float sc, float sc_hi, 
   const float2 lf = __ffma2_rn(hf, make_float2(-4194304.f, -4194304.f), __fmul2_rn(val, make_float2(sc, sc)));
   hi = make_int2(__float2int_rz(hf.x), __float2int_rz(hf.y));
   lo = make_uint2(__float2uint_rn(lf.x), __float2uint_rn(lf.y));
+}
+
+// box_deposit_s's words of two values at once.
+__device__ __forceinline__ void fixed_split2_s(float2 val, float sc, float sc_hi, int2& hi, int2& lo) {
+  const float2 t = __fmul2_rn(val, make_float2(sc_hi, sc_hi));
+  const float2 hf = make_float2(rintf(t.x), rintf(t.y));
+  const float2 lf = __ffma2_rn(hf, make_float2(-4194304.f, -4194304.f), __fmul2_rn(val, make_float2(sc, sc)));
+  hi = make_int2(__float2int_rz(hf.x), __float2int_rz(hf.y));
+  lo = make_int2(__float2int_rn(lf.x), __float2int_rn(lf.y));
 }
 
 }  // namespace e2e
