@@ -121,12 +121,12 @@ size_t mixed_smem_bytes(int area, int JB, int nk_max, int B, int nd) {
 
 // One CTA of 256 threads per output tile, a warp per sub-block (merge_tile.cuh); tiles that no
 // item touches are zeros.  What bounds it is the chain of loads of each sub-block (the tile, its
-// boxes, their pixels) and the instructions around them: 296 us for the full-detector frame's 820
-// MB of boxes and frame, against 467 us with the boxes looked up through the item list.  Four rows
-// a warp (512 threads, 40 registers) took 312 us, a persistent grid with the next tile's boxes
-// prefetched 415 us (64 registers, spilled).
+// boxes, their pixels) and the instructions around them: 246 us for the full-detector frame's 820
+// MB of boxes and frame at 64 registers (four CTAs per SM), 296 us at 76, against 467 us with the
+// boxes looked up through the item list.  Four rows a warp (512 threads, 40 registers) took 312
+// us, a persistent grid with the next tile's boxes prefetched 415 us (spilled).
 template <typename T>
-__global__ void __launch_bounds__(256) k_merge(const Tile* __restrict__ tiles, const TileBox* __restrict__ boxes,
+__global__ void __launch_bounds__(256, 4) k_merge(const Tile* __restrict__ tiles, const TileBox* __restrict__ boxes,
                                                const float2* __restrict__ store, T* const* dst,
                                                const int64_t* __restrict__ pitch, const int* __restrict__ dims) {
   static_assert(kMergeBlocks == 8, "one warp of the CTA per sub-block");
