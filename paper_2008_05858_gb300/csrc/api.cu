@@ -24,6 +24,7 @@
 #include "../../include/e2e_render.h"
 #include "e2e_device.cuh"
 #include "e2e_kernels.h"
+#include "ellip_moments.cuh"
 #include "poly_tables.cuh"
 #include "tail_coeffs.h"
 
@@ -68,6 +69,9 @@ struct Plan {
   int B = 1, DX = 0, DY = 0, JB = 1, NB = 8, max_area = 0, max_deg = 0, nk_max = 1;
   int B_adj = 1;      // run length of the adjoint (its FP32 sums run over one run)
   int poly = 0;       // separable kernel: polynomial pixel integrals (every sample's table is built)
+  int emom = 0;       // elliptical: rendered on run moments (every slice's nodes are built)
+  std::vector<EllGroup> egroups;  // its CTAs' items, in item order
+  EllGroup* d_egroups = nullptr;
   int far_tails = 0;  // separable kernel: every tail edge's argument within the cheaper rational's fit
   std::vector<Item> items;  // host copy
   int64_t store_elems = 0;
@@ -137,6 +141,7 @@ struct Model {
   int parent_coef_total = 0;
   int* d_fold = nullptr;  // first_sub | sub coef_off | parent coef_off | parent nc (adjoint folding)
   float4* d_stab = nullptr;  // per-sample tables of every slice (DevSlice::samples)
+  float* d_enodes = nullptr; // elliptical PSF: node tables of every slice (DevSlice::enodes), or null
   bool has_poly = false;     // ... followed by the polynomial pixel integrals (DevSlice::poly)
 };
 
@@ -357,6 +362,7 @@ void free_plan(Plan& p) {
   cudaFree(p.d_tile_of);
   cudaFree(p.d_grid_off);
   cudaFree(p.d_zero_tiles);
+  cudaFree(p.d_egroups);
   p = Plan{};
 }
 
@@ -375,6 +381,7 @@ void free_model(Model* m) {
   cudaFree(m->d_dims);
   cudaFree(m->d_fold);
   cudaFree(m->d_stab);
+  cudaFree(m->d_enodes);
   free_plan(m->plan);
 }
 
@@ -565,6 +572,58 @@ int plan_bands_and_tiles(Model* m) {
   return E2E_OK;
 }
 
+// Wavelength samples between two nodes of an elliptical slice's table (a multiple of 32), or 0
+// when its widths vary too fast or are too narrow: the cubic's error is 9/384 h^4 of the fourth
+// derivative in lt, and a pixel four widths from the centre changes at the rate 16 sigma'/sigma.
+int ellip_span(const e2e_order_slice& s) {
+  if (!ellip_moments_supported(s.K)) return 0;
+  const int n_jb = (s.n_lambda + 31) / 32;
+  double rate = 0.0;
+  for (const double* c : {s.sigma_x, s.sigma_y}) {
+    const double lo = quad_min(c);
+    if (lo < kEllMinSigma) return 0;
+    rate = std::max(rate, 16.0 * (std::fabs(c[1]) + 2.0 * std::fabs(c[2])) / lo);
+  }
+  const double h = 0.0455;  // (1e-7 * 384 / 9)^(1/4)
+  const double g = rate > 0.0 ? h / rate * s.n_lambda / 64.0 : (double)n_jb;
+  return g < 1.0 ? 0 : 32 * (int)std::min(g, (double)n_jb);
+}
+
+// Node tables of an elliptical model, rebuilt on the device whenever its widths change; without
+// them (a slice's widths, or no room) the model renders stamp by stamp.
+int build_ellip_nodes(Model* m) {
+  m->plan.emom = 0;
+  const int ns = (int)m->slices.size();
+  for (int i = 0; i < ns; ++i) m->dev[i].enodes = nullptr;
+  if (m->psf != E2E_PSF_ELLIPTICAL) return E2E_OK;
+  cudaFree(m->d_enodes);
+  m->d_enodes = nullptr;
+  int64_t total = 0;
+  int max_nodes = 0;
+  std::vector<int64_t> off(ns);
+  for (int i = 0; i < ns; ++i) {
+    const auto& s = m->slices[i].d;
+    const int span = ellip_span(s);
+    if (!span) return E2E_OK;
+    m->dev[i].espan = span;
+    const int n = (s.n_lambda + span - 1) / span + 3;
+    max_nodes = std::max(max_nodes, n);
+    off[i] = total;
+    total += n * ellip_node_floats(s.K);
+  }
+  if (cudaMalloc((void**)&m->d_enodes, (size_t)total * sizeof(float)) != cudaSuccess) {
+    cudaGetLastError();
+    m->d_enodes = nullptr;
+    return E2E_OK;
+  }
+  for (int i = 0; i < ns; ++i) m->dev[i].enodes = m->d_enodes + off[i];
+  E2E_CK(cudaMemcpy(m->d_slices, m->dev.data(), ns * sizeof(DevSlice), cudaMemcpyHostToDevice));
+  E2E_CK(launch_ellip_nodes(m->d_slices, ns, max_nodes, 0));
+  E2E_CK(cudaDeviceSynchronize());
+  m->plan.emom = 1;
+  return E2E_OK;
+}
+
 // Per-sample tables (mapping coefficients in s and PSF constants at each wavelength sample)
 // of every slice, rebuilt on the device whenever the model's coefficients change.
 int build_sample_tables(Model* m) {
@@ -621,6 +680,7 @@ int plan_model(Model* m) {
   const bool ellip = m->psf != E2E_PSF_SEPARABLE;  // item shape of the non-separable kernels
   if (ns == 0) return plan_bands_and_tiles(m);
   if (int rc0 = build_sample_tables(m); rc0 != E2E_OK) return rc0;
+  if (int rc0 = build_ellip_nodes(m); rc0 != E2E_OK) return rc0;
   // ---- device pass: exact window origins of every stamp
   std::vector<int64_t> task_off(ns + 1, 0), bb_off(ns + 1, 0);
   std::vector<int> n_jb(ns), n_k16(ns);
@@ -708,7 +768,7 @@ int plan_model(Model* m) {
 
   // ---- items: (32-sample blocks) x (16-point blocks); at most 16 warp tasks (<= 512 runs,
   // which keeps the fixed-point low words of a box below 2^31) and a box that fits on chip
-  for (int jb_cap = 8; jb_cap >= 1; jb_cap /= 2) {
+  for (int jb_cap = 8; jb_cap >= 1; P.emom ? P.emom = 0 : jb_cap /= 2) {
     int64_t store = 0;
     P.items.clear();
     P.groups.clear();
@@ -723,6 +783,10 @@ int plan_model(Model* m) {
         const int nrc = std::min(nrc_full, (KC * 16 + P.B - 1) / P.B);
         int JB = std::max(1, std::min(jb_cap, std::min((8 + nrc - 1) / nrc, 16 / nrc)));
         if (ellip) KC = JB = 1;  // <= 512 stamps: <= 512 deposits per box pixel
+        if (P.emom) {            // the slit in equal parts of at most kEllMaxSlit points
+          const int parts = (n_k16[i] * 16 + kEllMaxSlit - 1) / kEllMaxSlit;
+          KC = (n_k16[i] + parts - 1) / parts;
+        }
         P.JB = std::max(P.JB, JB);
         for (int b0 = 0; b0 < n_jb[i]; b0 += JB)
           for (int c0 = 0; c0 < n_k16[i]; c0 += KC) {
@@ -765,6 +829,7 @@ int plan_model(Model* m) {
       P.nk_max = std::max(P.nk_max, it.nk);
     }
     P.smem = m->psf == E2E_PSF_TABLE ? table_smem_bytes(P.max_area, P.nk_max, P.max_deg + 1)
+             : P.emom ? ellip_moment_smem(m->Ks.back(), P.max_area, P.nk_max, P.max_deg + 1)
              : ellip ? ellip_smem_bytes(P.max_area, P.nk_max, P.max_deg + 1, m->Ks.empty() ? 15 : m->Ks.front())
              : P.poly ? poly_smem_bytes(P.max_area, P.JB, P.nk_max, P.max_deg + 1)
                      : mixed_smem_bytes(P.max_area, P.JB, P.nk_max, P.B, P.max_deg + 1);
@@ -772,12 +837,28 @@ int plan_model(Model* m) {
     // would not fill the GPU gets items of one 32-sample block (a sample octet per warp)
     const bool thin = P.poly && jb_cap > 1 && P.JB > 1 && (int)P.items.size() < kPolyWave;
     if ((int)P.smem + kStaticSmemReserve <= optin && !thin) break;
-    if (jb_cap == 1)
+    if (jb_cap == 1 && !P.emom)
       return fail(E2E_EINVAL, "trace footprint of a work item exceeds on-chip memory (area " +
                                   std::to_string(P.max_area) + " px)");
   }
   P.NB = 1;
-  return plan_bands_and_tiles(m);
+  if (int rc1 = plan_bands_and_tiles(m); rc1 != E2E_OK) return rc1;
+  if (P.emom) {
+    // a CTA's items: neighbours of one slice, interval and band, at most four (each CTA loads its
+    // interval's nodes once), fewer where the GPU would run out of CTAs
+    const int cap = std::max(1, std::min(4, (int)P.items.size() / (152 * 4)));
+    for (size_t s = 0; s < P.seg_count.size(); ++s)
+      for (int n = P.seg_first[s]; n < P.seg_first[s] + P.seg_count[s]; ++n) {
+        const Item& it = P.items[n];
+        const int v = it.j0 / m->dev[it.slice].espan;
+        EllGroup* g = P.egroups.empty() ? nullptr : &P.egroups.back();
+        if (!g || n == P.seg_first[s] || g->count == cap || P.items[n - 1].slice != it.slice || g->interval != v)
+          P.egroups.push_back(EllGroup{n, 0, v, 0});
+        P.egroups.back().count++;
+      }
+    return upload(&P.d_egroups, P.egroups.data(), P.egroups.size());
+  }
+  return E2E_OK;
 }
 
 // ------------------------------------------------------------------ render
@@ -881,6 +962,15 @@ cudaError_t launch_items(e2e_ctx* ctx, Model* m, int K, int first, int count, co
   if (m->psf == E2E_PSF_TABLE)
     return launch_render_table(K, m->d_slices, m->d_ts, m->d_T32, m->d_field, d_table, m->d_u,
                                P.d_items + first, count, store, P.nk_max, P.max_deg, P.smem, st, ctx->d_err);
+  if (P.emom) {
+    auto at = [&](int n) {
+      return std::lower_bound(P.egroups.begin(), P.egroups.end(), n,
+                              [](const EllGroup& g, int i) { return g.first < i; }) - P.egroups.begin();
+    };
+    const int g0 = (int)at(first), g1 = (int)at(first + count);
+    return launch_ellip_moments(K, m->d_slices, d_table, m->d_u, P.d_items, P.d_egroups + g0, g1 - g0, store,
+                                P.nk_max, P.max_deg, P.smem, st, ctx->d_err);
+  }
   if (m->psf == E2E_PSF_ELLIPTICAL)
     return launch_render_ellip(K, m->d_slices, d_table, m->d_u, P.d_items + first, count, store, P.nk_max,
                                P.max_deg, P.smem, st, ctx->d_err);

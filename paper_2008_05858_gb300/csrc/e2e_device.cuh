@@ -35,6 +35,10 @@ struct DevSlice {
   // polynomial pixel integrals (poly_tables.cuh), or null: for wavelength sample j, the
   // 4 poly_role_f4(K) float4 at poly + j 4 poly_role_f4(K), one block per role 2 half + axis
   const float4* poly;
+  // elliptical PSF: node tables of the pixel integrals' coefficients (ellip_moments.cuh), or null,
+  // and the wavelength samples between two nodes
+  const float* enodes;
+  int32_t espan, pad;
 };
 
 // A mixed-path work item: a block of wavelength samples x a block of slit points of one

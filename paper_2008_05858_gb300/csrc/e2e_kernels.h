@@ -59,6 +59,15 @@ size_t ellip_smem_bytes(int area, int nk_max, int nd, int k_min);
 cudaError_t launch_render_ellip(int K, const DevSlice* slices, const double* const* flux_tab, const double* u_all,
                                 const Item* items, int n_items, float2* store, int nk_max, int max_deg, size_t smem,
                                 cudaStream_t st, int* err = nullptr);
+// The elliptical render on run moments (render_ellip_moments.cu; DevSlice::enodes set).
+struct EllGroup;
+bool ellip_moments_supported(int K);
+size_t ellip_moment_smem(int K, int area, int nk_max, int nd);
+int64_t ellip_node_floats(int K);
+cudaError_t launch_ellip_nodes(const DevSlice* slices, int n_slices, int max_nodes, cudaStream_t st);
+cudaError_t launch_ellip_moments(int K, const DevSlice* slices, const double* const* flux_tab, const double* u_all,
+                                 const Item* items, const EllGroup* groups, int n_groups, float2* store, int nk_max,
+                                 int max_deg, size_t smem, cudaStream_t st, int* err = nullptr);
 cudaError_t launch_render_fp64_ellip(int K, int n_slices, int64_t max_stamps, const DevSlice* slices,
                                      const double* const* flux_tab, const double* u_all, double* const* acc,
                                      const int64_t* pitch, cudaStream_t st);
