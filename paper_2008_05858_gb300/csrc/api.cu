@@ -1522,7 +1522,7 @@ int e2e_load_model(e2e_ctx* ctx, const e2e_model_desc* desc_in, uint64_t* model_
       const DevSlice& v = ds[i];
       for (int c = 0; c < 2; ++c) {
         const double* co = c ? v.cy : v.cx;
-        float* o = cf.data() + i * nf + c * (E2E_MAXC + 2);
+        float* o = cf.data() + i * nf + c * kPhotonCoord;
         double qb = 0.0, sb = 0.0;
         for (int a = 0; a <= v.degree; ++a)
           for (int b = 0; a + b <= v.degree; ++b) {
@@ -1534,7 +1534,7 @@ int e2e_load_model(e2e_ctx* ctx, const e2e_model_desc* desc_in, uint64_t* model_
         o[E2E_MAXC] = (float)qb;
         o[E2E_MAXC + 1] = (float)sb;
       }
-      float* e = cf.data() + i * nf + 2 * (E2E_MAXC + 2);  // sigma_x, sigma_y, slit-weight total
+      float* e = cf.data() + i * nf + 2 * kPhotonCoord;  // sigma_x, sigma_y, slit-weight total
       for (int k = 0; k < 3; ++k) {
         e[k] = (float)v.sx[k];
         e[3 + k] = (float)v.sy[k];

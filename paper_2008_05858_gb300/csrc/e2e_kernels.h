@@ -107,6 +107,7 @@ cudaError_t launch_photon_bins(const DevSlice* slices, int n_slices, const doubl
                                int4* anchors, int* bin_slice, cudaStream_t st);
 constexpr int kPhotonGuide = 1 << 20;  // entries of the photon -> bin guide table (+1)
 cudaError_t launch_photon_guide(const uint64_t* offsets, int64_t n_bins, int64_t* guide, cudaStream_t st);
+constexpr int kPhotonCoord = 48;  // floats per coordinate of a slice's FP32 copy (photon.cu), 16-byte rows
 size_t photon_coef_floats();
 size_t scan_scratch_elems(int64_t n);
 cudaError_t launch_scan_exclusive(const uint64_t* in, uint64_t* out, int64_t n, uint64_t* scratch, cudaStream_t st);

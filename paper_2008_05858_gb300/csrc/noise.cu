@@ -27,6 +27,7 @@
 // (the common case) runs in two passes: the first issues no FP64 instruction and lists the
 // pairs it cannot decide, the second redoes only those pairs in FP64; FP64 electrons and
 // expected values (no shot noise) take the one-pass kernel, which redoes draws inline.
+#include <cmath>
 #include <cstdint>
 
 #include "e2e_kernels.h"
@@ -198,30 +199,19 @@ __device__ __forceinline__ void split_src(TI v, float& h, float& l) {
   }
 }
 
-// Poisson count of mean (lh, ll) +- le decided in FP32, or -1.
-__device__ __forceinline__ int count_f32(float lh, float ll, float le, uint64_t seed, uint32_t q, uint32_t d,
-                                         uint32_t stream) {
-  if (lh + le <= 0.f) return 0;  // the mean is <= 0: no photons
-  if (lh - le <= 0.f) return -1;
-  if (lh + le < 10.f) return inversion_f32(lh, 6e-8f + le / lh, seed, q, d, stream);
-  if (lh - le < 10.f) return -1;  // which sampler applies is too close to call
-  float Lf = floorf(lh), frac = (lh - Lf) + ll;
-  if (frac < 0.f) {
-    Lf -= 1.f;
-    frac += 1.f;
-  } else if (frac >= 1.f) {
-    Lf += 1.f;
-    frac -= 1.f;
-  }
-  return ptrs_f32(Lf, frac, le, seed, q, d, stream);
-}
+// The ADU conversion's constants to more than FP32: 1 / gain less its FP32 value, bias + 1/2 as a
+// whole number and the rest, and a bound on what the two leave out.
+struct AduArgs {
+  float inv_gain_lo, bias_whole, bias_frac, bias_err;
+};
 
 template <typename TI, typename TO>
 __global__ void __launch_bounds__(256, 8) k_noise_first(const NoiseArgs a, const TI* __restrict__ src,
                                                      int64_t src_pitch, const float* __restrict__ R32,
                                                      const float* __restrict__ R32lo, TO* dst, int64_t dst_pitch,
                                                      int H, int W, int det, unsigned* __restrict__ list,
-                                                     unsigned* __restrict__ n_list, float dark_lo) {
+                                                     unsigned* __restrict__ n_list, float dark_lo,
+                                                     const AduArgs ad) {
   const int half = (W + 1) / 2;
   const int n = H * half;  // < 2^31 (the launcher checks)
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
@@ -254,17 +244,23 @@ __global__ void __launch_bounds__(256, 8) k_noise_first(const NoiseArgs a, const
         v[0] = e0;
         v[1] = e1;
       } else {  // ADU = clamp(floor((bias + E / gain) + 1/2)), decided exactly or deferred
-        const float ig = a.inv_gain32, bias = a.bias32;
-        const float tt[2] = {fmaf(e0, ig, bias) + 0.5f, fmaf(e1, ig, bias) + 0.5f};
-        const float ee[2] = {e0, e1};
+        // N / gain as a product with its FMA error term, its whole part and the bias's set aside:
+        // only a fraction and the small terms (read-out noise, cross-talk) are rounded, so the
+        // margin does not grow with the signal (rounded as one FP32 number, a 1e4 e- pixel's was
+        // 8e-3 ADU and one pair in sixty of a bright trace was redone in FP64)
+        const float ig = a.inv_gain32;
 #pragma unroll
         for (int s2 = 0; s2 < 2; ++s2) {
-          const float xn = fabsf(xt) * (s2 ? nf0 : nf1);
-          const float mt = fmaf(fmaf(fabsf(ee[s2]), 4e-7f, fmaf(fabsf(ron), eg, xn * 2e-7f)), ig,
-                                fmaf(fabsf(tt[s2]), 4e-7f, 1e-6f));
-          const float lo = floorf(tt[s2] - mt);
-          defer = defer || (lo != floorf(tt[s2] + mt));
-          v[s2] = fminf(fmaxf(lo, 0.f), a.sat32);
+          const float nf = s2 ? nf1 : nf0, xn = xt * (s2 ? nf0 : (two ? nf1 : 0.f));
+          const float ph = nf * ig, pe = fmaf(nf, ig, -ph) + nf * ad.inv_gain_lo;
+          const float whole = floorf(ph);
+          const float small = fmaf(ron, s2 ? g1 : g0, xn) * ig;
+          const float f = ((ph - whole) + ad.bias_frac) + (pe + small);
+          const float mt = fmaf(fmaf(fabsf(xn), 4e-7f, fabsf(ron) * eg), ig, fmaf(fabsf(small) + fabsf(f), 4e-7f, 1e-6f)) +
+                           ad.bias_err + (nf < 8388608.f && fabsf(ph) < 8388608.f ? 0.f : nf * ig);
+          const float lo = floorf(f - mt);
+          defer = defer || (lo != floorf(f + mt));
+          v[s2] = fminf(fmaxf((whole + ad.bias_whole) + lo, 0.f), a.sat32);
         }
       }
     }
@@ -343,7 +339,7 @@ cudaError_t launch_prnu_map(double* R, float* R32, float* R32lo, int H, int W, i
 }
 
 template <typename TI, typename TO>
-static cudaError_t launch_two_pass_t(const NoiseArgs& a, float dark_lo, const void* src, int64_t sp, const double* R,
+static cudaError_t launch_two_pass_t(const NoiseArgs& a, float dark_lo, const AduArgs& ad, const void* src, int64_t sp, const double* R,
                                      const float* R32, const float* R32lo, void* dst, int64_t dp, int H, int W,
                                      int det, unsigned* list, unsigned* n_list, cudaStream_t st) {
   const int64_t n = (int64_t)H * ((W + 1) / 2);
@@ -352,7 +348,7 @@ static cudaError_t launch_two_pass_t(const NoiseArgs& a, float dark_lo, const vo
   cudaError_t e = cudaMemsetAsync(n_list, 0, sizeof(unsigned), st);
   if (e != cudaSuccess) return e;
   k_noise_first<TI, TO><<<(unsigned)grid_blocks(n), 256, 0, st>>>(a, (const TI*)src, sp, R32, R32lo, (TO*)dst, dp, H,
-                                                                   W, det, list, n_list, dark_lo);
+                                                                   W, det, list, n_list, dark_lo, ad);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   k_noise_redo<TI, TO><<<152 * 4, 256, 0, st>>>(a, (const TI*)src, sp, R, (TO*)dst, dp, H, W, det, list, n_list);
@@ -368,9 +364,14 @@ cudaError_t launch_noise_two_pass(uint64_t seed, uint64_t pattern_seed, double d
                     gain,        bias,         saturation,  1,           (float)dark, (float)(1.0 / gain),
                     (float)ron,  (float)xtalk, (float)bias, (float)saturation};
   const float dark_lo = (float)(dark - (double)(float)dark);
+  AduArgs ad;
+  ad.inv_gain_lo = (float)(1.0 / gain - (double)a.inv_gain32);
+  ad.bias_whole = (float)std::floor(bias + 0.5);
+  ad.bias_frac = (float)(bias + 0.5 - (double)ad.bias_whole);
+  ad.bias_err = (float)(1.01 * std::fabs(bias + 0.5 - (double)ad.bias_whole - (double)ad.bias_frac));
 #define E2E_N(SI, TI, DI, TO) \
   if (src_dtype == SI && dst_dtype == DI)  \
-    return launch_two_pass_t<TI, TO>(a, dark_lo, src, src_pitch, R, R32, R32lo, dst, dst_pitch, H, W, det, list, n_list, st);
+    return launch_two_pass_t<TI, TO>(a, dark_lo, ad, src, src_pitch, R, R32, R32lo, dst, dst_pitch, H, W, det, list, n_list, st);
   E2E_N(0, float, 0, float) E2E_N(0, float, 2, uint16_t) E2E_N(1, double, 0, float) E2E_N(1, double, 2, uint16_t)
 #undef E2E_N
   return cudaErrorInvalidValue;

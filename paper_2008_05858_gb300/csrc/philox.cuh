@@ -125,8 +125,8 @@ __device__ __forceinline__ void normal_pair_f32(uint64_t seed, uint32_t q, uint3
 // Poisson draw with the exact function's integer result, from FP32 arithmetic whenever its
 // error bound decides every comparison (see the file comment).
 // Sequential-inversion Poisson draw in FP32 for a mean l known to relative accuracy lrel:
-// F_k within F (8.4e-7 + 2.4e-7 k) of the FP64 sums plus F (k + l) lrel for the mean's own
-// error, u within 2^-23 relative; all bounds doubled.  Returns the count, or -1 when some
+// F_k within F (8.4e-7 + 3.6e-7 k) of the FP64 sums plus F (k + l) lrel for the mean's own
+// error, u within 2^-23 relative; the bounds taken twice as large or more.  Returns the count, or -1 when some
 // comparison is too close to call (the caller then draws exactly).
 static __device__ int inversion_f32(float l, float lrel, uint64_t seed, uint32_t q, uint32_t d, uint32_t stream) {
   const uint4 w = rng_block(seed, q, d, 0, stream);
@@ -136,8 +136,8 @@ static __device__ int inversion_f32(float l, float lrel, uint64_t seed, uint32_t
     const float rel = fmaf(1e-6f, (float)k, 4e-6f) + 2.f * ((float)k + l) * lrel;
     const float tol = fmaf(F, rel, fmaf(u, 2.5e-7f, 1e-12f));
     const float diff = u - F;
-    if (diff > tol) {  // u > F_k: one more
-      p = p * (l / (float)(k + 1));
+    if (diff > tol) {  // u > F_k: one more (the quick division's 2 ulp are in the bound)
+      p = p * __fdividef(l, (float)(k + 1));
       F = F + p;
       continue;
     }
@@ -258,15 +258,18 @@ static __device__ int ptrs_f32(float Lf, float frac, float le, uint64_t seed, ui
   const float sl = sqrtf(l);
   const float b = fmaf(2.53f, sl, 0.931f);
   const float a = fmaf(0.02483f, b, -0.059f);
-  const float vr = 0.9277f - 3.6224f / (b - 2.f);
-  const float lia = logf(1.1239f + 1.1328f / (b - 3.4f));  // ln(1 / alpha)
+  const float vr = 0.9277f - __fdividef(3.6224f, b - 2.f);  // quick divisions: 2 ulp, in the margins below
   for (uint32_t i = 0; i < 64; ++i) {
     const uint4 w = rng_block(seed, q, d, i, stream);
-    const float U = uni53_f32(w.x, w.y) - 0.5f, V = uni53_f32(w.z, w.w);
+    // u - 1/2 from the words, within 2^-23 of itself (not of 1/2): a bright pixel's T is hundreds
+    const float U = fmaf((float)((int)(w.x >> 5) - 0x4000000), 0x1p-27f,
+                         fmaf(__uint2float_rn(w.y >> 6), 0x1p-53f, 0x1p-54f));
+    const float V = uni53_f32(w.z, w.w);
     const float us = 0.5f - fabsf(U);
-    const float T = 2.f * a / us + b;
+    const float T = __fdividef(2.f * a, us) + b;
     const float y = T * U;
-    const float yerr = fabsf(T) * fmaf(fabsf(U), fmaf(3e-7f, 1.f / us, 4e-6f), 2e-7f) + 1e-6f;
+    // T within (6e-7 + 2e-7 / us) of itself (b 1.5e-7, a 3e-7, the division 2.4e-7, us 9e-8 absolute)
+    const float yerr = fabsf(y) * fmaf(3e-7f, __fdividef(1.f, us), 1.5e-6f) + 1e-6f;
     const float xr = (y + frac) + 0.43f;
     const float xe = yerr + fmaf(fabsf(xr), 2.5e-7f, 1e-7f) + le;
     const float kr = floorf(xr - xe);
@@ -280,6 +283,7 @@ static __device__ int ptrs_f32(float Lf, float frac, float le, uint64_t seed, ui
     if (d1t && d2t) continue;
     if (!(d1f || d2f)) return -1;
     // slow acceptance: ln V + ln(1/alpha) - ln(a / us^2 + b) <= ln p(k)
+    const float lia = logf(1.1239f + 1.1328f / (b - 3.4f));  // ln(1 / alpha)
     const float lhs = logf(V) + lia - logf(a / (us * us) + b);
     const float elhs = fmaf(1e-6f, fabsf(lhs), 6e-6f) + 3e-7f / us;
     float erhs;
@@ -289,6 +293,24 @@ static __device__ int ptrs_f32(float Lf, float frac, float le, uint64_t seed, ui
     return -1;
   }
   return -1;
+}
+
+// Poisson count of mean (lh, ll) +- le decided in FP32, or -1.
+__device__ __forceinline__ int count_f32(float lh, float ll, float le, uint64_t seed, uint32_t q, uint32_t d,
+                                         uint32_t stream) {
+  if (lh + le <= 0.f) return 0;  // the mean is <= 0: no photons
+  if (lh - le <= 0.f) return -1;
+  if (lh + le < 10.f) return inversion_f32(lh, 6e-8f + le / lh, seed, q, d, stream);
+  if (lh - le < 10.f) return -1;  // which sampler applies is too close to call
+  float Lf = floorf(lh), frac = (lh - Lf) + ll;
+  if (frac < 0.f) {
+    Lf -= 1.f;
+    frac += 1.f;
+  } else if (frac >= 1.f) {
+    Lf += 1.f;
+    frac -= 1.f;
+  }
+  return ptrs_f32(Lf, frac, le, seed, q, d, stream);
 }
 
 // A Poisson count: k when the FP32 draw decided it, else (k < 0) the FP64 value x.

@@ -29,12 +29,13 @@
 namespace e2e {
 
 // FP32 copy of a slice's mapping coefficients and the bounds its fast path uses: per
-// coordinate 45 coefficients, then sum_a a |c_a0| (bounds the divided difference of the b = 0
+// coordinate (kPhotonCoord floats) 45 coefficients, then sum_a a |c_a0| (bounds the divided difference of the b = 0
 // polynomial) and sum_{b >= 1} |c_ab| (bounds the slit terms); then the PSF-width
 // coefficients sigma_x[0..2], sigma_y[0..2], the slit-weight total and one pad, all rounded
 // to FP32 once on the host.
-constexpr int kCfExtra = 2 * (E2E_MAXC + 2);
+constexpr int kCfExtra = 2 * kPhotonCoord;
 constexpr int kCf = kCfExtra + 8;
+static_assert(E2E_MAXC + 2 <= kPhotonCoord && kPhotonCoord % 4 == 0 && kCf % 4 == 0, "16-byte rows");
 
 // Per bin: the photon count, and the bin centre's position at s = 0 in FP64, split into the
 // nearest integer and an FP32 remainder (the anchor the FP32 fast path adds small terms to).
@@ -54,7 +55,13 @@ __global__ void __launch_bounds__(256) k_photon_bins(const DevSlice* __restrict_
     bin_slice[b] = lo;
     const int j = (int)(b - bin_off[lo]);
     const double lam = __dmul_rn(__dmul_rn(flux_tab[S.flux_slot][j], S.dlam), usum[lo]);
-    counts[b] = (uint64_t)poisson_filtered(lam, seed, (uint32_t)j, (uint32_t)S.index, 4);
+    // decided in FP32 (the sampler of the noise stage's first pass), else drawn in FP64: with the
+    // FP64 steps of poisson_filtered in every warp's way 2e6 bins of 50 photons took 1.73 ms, not 0.24
+    const float lh = (float)lam;
+    int k = -1;
+    if (lh < 8388608.f)
+      k = count_f32(lh, (float)(lam - (double)lh), fmaf(1e-13f, lh, 1e-37f), seed, (uint32_t)j, (uint32_t)S.index, 4);
+    counts[b] = k >= 0 ? (uint64_t)k : (uint64_t)poisson_draw(lam, seed, (uint32_t)j, (uint32_t)S.index, 4);
     const double ltj = norm_sample(j, S.n_lambda);
     const double X0 = poly_lt_for_b(S.cx, S.degree, 0, ltj), Y0 = poly_lt_for_b(S.cy, S.degree, 0, ltj);
     const bool ok = fabs(X0) < 1e9 && fabs(Y0) < 1e9;
@@ -199,8 +206,18 @@ __device__ void photon_exact(const DevSlice& S, const double* __restrict__ C, do
 // difference, so no large terms cancel) plus the slit terms sum_{b>=1} P_b(lt) s^b.  D is the
 // slice's degree, a template parameter so that only its terms are evaluated.
 template <int D>
-__device__ __forceinline__ float photon_offset(const float* cf, float lt, float ltj, float delta, float s,
+__device__ __forceinline__ float photon_offset(const float* row, float lt, float ltj, float delta, float s,
                                                float& mag) {
+  constexpr int NC4 = ((D + 1) * (D + 2) / 2 + 3) / 4;
+  float cf[4 * NC4];
+#pragma unroll
+  for (int q = 0; q < NC4; ++q) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(row) + q);
+    cf[4 * q] = v.x;
+    cf[4 * q + 1] = v.y;
+    cf[4 * q + 2] = v.z;
+    cf[4 * q + 3] = v.w;
+  }
   float q[8];
 #pragma unroll
   for (int a = 0; a < 8; ++a) q[a] = 0.f;
@@ -224,7 +241,7 @@ __device__ __forceinline__ float photon_offset(const float* cf, float lt, float 
     sb = fmaf(sb, s, pb);
   }
   sb *= s;
-  mag = fabsf(delta) * cf[E2E_MAXC] + cf[E2E_MAXC + 1];
+  mag = fabsf(delta) * row[E2E_MAXC] + row[E2E_MAXC + 1];
   return fmaf(delta, Q, sb);
 }
 
@@ -235,13 +252,13 @@ __device__ __forceinline__ void photon_offsets(int d, const float* cf, float lt,
 #define E2E_PO(D)                                                                   \
   case D:                                                                           \
     ox = photon_offset<D>(cf, lt, ltj, delta, s, mx);                               \
-    oy = photon_offset<D>(cf + E2E_MAXC + 2, lt, ltj, delta, s, my);                \
+    oy = photon_offset<D>(cf + kPhotonCoord, lt, ltj, delta, s, my);                \
     return;
     E2E_PO(0) E2E_PO(1) E2E_PO(2) E2E_PO(3) E2E_PO(4) E2E_PO(5) E2E_PO(6) E2E_PO(7)
 #undef E2E_PO
     default:
       ox = photon_offset<8>(cf, lt, ltj, delta, s, mx);
-      oy = photon_offset<8>(cf + E2E_MAXC + 2, lt, ltj, delta, s, my);
+      oy = photon_offset<8>(cf + kPhotonCoord, lt, ltj, delta, s, my);
   }
 }
 
@@ -261,13 +278,16 @@ __global__ void __launch_bounds__(256, E2E_PHOTON_MIN_BLOCKS) k_photons(const De
                                                  const int64_t* __restrict__ guide) {
   const int64_t nb = bin_off[n_slices];
   const uint64_t total = offsets[nb];
+  // floor(p G / total) by the high word of p G times floor(2^64 / total): it or one less (a 64-bit
+  // division per photon was an eighth of the instructions), so the search spans two guide steps
+  const uint64_t inv_total = total > 1 ? ~0ull / total : 0;
   for (uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; p < total;
        p += (uint64_t)gridDim.x * blockDim.x) {
     int64_t lo = 0, hi = nb - 1;
     if (total < kGuidedPhotons) {
-      const uint64_t g = p * kPhotonGuide / total;  // g < G since p < total
+      const int g = (int)__umul64hi(p * kPhotonGuide, inv_total);  // <= floor(p G / total) < G
       lo = guide[g];
-      hi = guide[g + 1];
+      hi = guide[min(g + 2, kPhotonGuide)];
     }
     const int64_t b = photon_bin(offsets, p, lo, hi);
     const int sl = bin_slice[b];
@@ -296,10 +316,13 @@ __global__ void __launch_bounds__(256, E2E_PHOTON_MIN_BLOCKS) k_photons(const De
       if (k0 < S.n_slit - 1 && !(C32[k0] - cu > tol)) exact = true;
       if (k0 > 0 && !(cu - C32[k0 - 1] > tol)) exact = true;
       const float n = (float)S.n_lambda, ns = (float)S.n_slit;
-      const float delta = (2.f * uni53_f32(wa.x, wa.y) - 1.f) / n;
-      const float ltj = (float)(2 * (int)j + 1 - S.n_lambda) / n;
+      // (quick divisions: 2 ulp each, at most 5e-6 of the slit terms through lt and s, inside the
+      // 1e-5 of the bounds below; seven full divisions were 70 of 824 instructions)
+      const float inv_n = __fdividef(1.f, n), inv_ns = __fdividef(1.f, ns);
+      const float delta = (2.f * uni53_f32(wa.x, wa.y) - 1.f) * inv_n;
+      const float ltj = (float)(2 * (int)j + 1 - S.n_lambda) * inv_n;
       const float lt = ltj + delta;
-      const float s = (2.f * ((float)k0 + uni53_f32(wa.z, wa.w)) - ns) / ns;
+      const float s = (2.f * ((float)k0 + uni53_f32(wa.z, wa.w)) - ns) * inv_ns;
       float z1, z2, eg;
       normal_pair_f32_ctr(seed, j, si, pp, 7, z1, z2, eg);
       const float sx = fmaf(fmaf(ce[2], lt, ce[1]), lt, ce[0]);
@@ -309,8 +332,9 @@ __global__ void __launch_bounds__(256, E2E_PHOTON_MIN_BLOCKS) k_photons(const De
       ox += sx * z1;
       oy += sy * z2;
       const float rx = __int_as_float(an.y) + ox + 0.5f, ry = __int_as_float(an.w) + oy + 0.5f;
-      const float ein = 4e-7f * ((cf[E2E_MAXC] / n) + (float)S.degree * cf[E2E_MAXC + 1] / ns);
-      const float einy = 4e-7f * ((cf[2 * E2E_MAXC + 2] / n) + (float)S.degree * cf[2 * E2E_MAXC + 3] / ns);
+      const float* cy = cf + kPhotonCoord;
+      const float ein = 4e-7f * (cf[E2E_MAXC] * inv_n + (float)S.degree * cf[E2E_MAXC + 1] * inv_ns);
+      const float einy = 4e-7f * (cy[E2E_MAXC] * inv_n + (float)S.degree * cy[E2E_MAXC + 1] * inv_ns);
       const float ex = 1e-5f * (mx + fabsf(sx * z1) + 1.f) + ein + 1.5f * sx * eg;
       const float ey = 1e-5f * (my + fabsf(sy * z2) + 1.f) + einy + 1.5f * sy * eg;
       const float kx = floorf(rx - ex), ky = floorf(ry - ey);
