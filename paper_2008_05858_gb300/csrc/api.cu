@@ -69,6 +69,7 @@ struct Plan {
   int B = 1, DX = 0, DY = 0, JB = 1, NB = 8, max_area = 0, max_deg = 0, nk_max = 1;
   int B_adj = 1;      // run length of the adjoint (its FP32 sums run over one run)
   int poly = 0;       // separable kernel: polynomial pixel integrals (every sample's table is built)
+  int tcap = 0, tcells = 0;  // tabulated PSF: stamps a CTA stages at a time; most phase cells of a slice
   int emom = 0;       // elliptical: rendered on run moments (every slice's nodes are built)
   std::vector<EllGroup> egroups;  // its CTAs' items, in item order
   EllGroup* d_egroups = nullptr;
@@ -828,7 +829,12 @@ int plan_model(Model* m) {
       P.max_area = std::max(P.max_area, it.bw * it.bh);
       P.nk_max = std::max(P.nk_max, it.nk);
     }
-    P.smem = m->psf == E2E_PSF_TABLE ? table_smem_bytes(P.max_area, P.nk_max, P.max_deg + 1)
+    for (auto& s : m->slices) {
+      const int c = (int)s.d.map_oversample + (s.d.map_size % 2 == 0 ? 1 : 0);  // phase cells per axis
+      if (m->psf == E2E_PSF_TABLE) P.tcells = std::max(P.tcells, c * c);
+    }
+    P.smem = m->psf == E2E_PSF_TABLE ? table_smem_bytes(P.max_area, P.nk_max, P.max_deg + 1, P.tcells,
+                                                        (size_t)optin - kStaticSmemReserve, &P.tcap)
              : P.emom ? ellip_moment_smem(m->Ks.back(), P.max_area, P.nk_max, P.max_deg + 1)
              : ellip ? ellip_smem_bytes(P.max_area, P.nk_max, P.max_deg + 1, m->Ks.empty() ? 15 : m->Ks.front())
              : P.poly ? poly_smem_bytes(P.max_area, P.JB, P.nk_max, P.max_deg + 1)
@@ -961,7 +967,8 @@ cudaError_t launch_items(e2e_ctx* ctx, Model* m, int K, int first, int count, co
   const Plan& P = m->plan;
   if (m->psf == E2E_PSF_TABLE)
     return launch_render_table(K, m->d_slices, m->d_ts, m->d_T32, m->d_field, d_table, m->d_u,
-                               P.d_items + first, count, store, P.nk_max, P.max_deg, P.smem, st, ctx->d_err);
+                               P.d_items + first, count, store, P.nk_max, P.max_deg, P.tcap, P.tcells, P.smem, st,
+                               ctx->d_err);
   if (P.emom) {
     auto at = [&](int n) {
       return std::lower_bound(P.egroups.begin(), P.egroups.end(), n,

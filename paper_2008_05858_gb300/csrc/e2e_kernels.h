@@ -86,10 +86,12 @@ cudaError_t launch_noise(uint64_t seed, uint64_t pattern_seed, double dark, doub
 
 cudaError_t launch_epsf_build(const TableSlice* ts, int n_slices, int max_field, int max_cells, const double* maps,
                               double* norms, double* T64, float* T32, cudaStream_t st);
-size_t table_smem_bytes(int area, int nk_max, int nd);
+// shared memory of the table kernel, and the stamps it stages at a time (*cap): as many as fit in limit
+size_t table_smem_bytes(int area, int nk_max, int nd, int cells, size_t limit, int* cap);
 cudaError_t launch_render_table(int K, const DevSlice* slices, const TableSlice* ts, const float* T32,
                                 const double* field_lt, const double* const* flux_tab, const double* u_all,
-                                const Item* items, int n_items, float2* store, int nk_max, int max_deg, size_t smem,
+                                const Item* items, int n_items, float2* store, int nk_max, int max_deg, int cap,
+                                int cells, size_t smem,
                                 cudaStream_t st, int* err = nullptr);
 cudaError_t launch_render_fp64_table(int K, int n_slices, int64_t max_stamps, const DevSlice* slices,
                                      const TableSlice* ts, const double* T64, const double* field_lt,

@@ -31,7 +31,7 @@ namespace e2e {
 constexpr int kPThreads = 128;
 constexpr int kPWarps = kPThreads / 32;
 constexpr int kNoStamp = 1 << 30;       // window centre of a stamp that deposits nothing
-// deposit_split2's bound on the high word, over the largest pixel integral of a PSF of widths
+// fixed_split2_small's bound on the high word, over the largest pixel integral of a PSF of widths
 // kPolyMinSigma = 1 (erf(1 / sqrt 8)^2 = 0.1466)
 constexpr float kSmallDeposit = 4190000.f / 0.147f;
 constexpr int kPQuad = 36;             // floats per quad and stamp of the exchange (4 mod 32: see below)
@@ -69,20 +69,6 @@ struct PolyLayout {
 // The two lane quadrants along an axis of R tile pixels: the first takes [0, quad_span), the
 // second the rest.
 __host__ __device__ constexpr int quad_span(int R) { return (R + 1) / 2; }
-
-// The fixed-point words of two deposits whose scaled values stay below 2^44 (their high words
-// below 2^22): fixed_split2 (mixed_common.cuh) with both words rounded to nearest by adding
-// 1.5 * 2^23 and read off the mantissa, the low word signed.  No conversions: on the quarter-rate
-// pipe they took a third of a flush.
-__device__ __forceinline__ void deposit_split2(float2 val, float sc, float sc_hi, int2& hi, int2& lo) {
-  constexpr float kMagic = 12582912.f;
-  const float2 m = make_float2(kMagic, kMagic);
-  const float2 h = __ffma2_rn(val, make_float2(sc_hi, sc_hi), m);
-  const float2 hf = __fadd2_rn(h, neg2(m));
-  const float2 l = __fadd2_rn(__ffma2_rn(hf, make_float2(-4194304.f, -4194304.f), __fmul2_rn(val, make_float2(sc, sc))), m);
-  hi = make_int2(__float_as_int(h.x) - 0x4B400000, __float_as_int(h.y) - 0x4B400000);
-  lo = make_int2(__float_as_int(l.x) - 0x4B400000, __float_as_int(l.y) - 0x4B400000);
-}
 
 // CHECK: debug build of the same kernel, counting into a.err every deposit the plan did not
 // foresee.
@@ -203,7 +189,7 @@ __global__ void __launch_bounds__(kPThreads, 4) k_render_poly(const MixedArgs a)
     int parity = 0;
     for (int k0 = 0; k0 < it.nk; k0 += 16) {
       const int nk = min(16, it.nk - k0);
-      bool small;  // every deposit of these stamps' tiles stays below 2^44 units (deposit_split2)
+      bool small;  // every deposit of these stamps' tiles stays below 2^44 units (fixed_split2_small)
       // map 16 slit points, a quarter per lane; the tile origin of each run of B of them is the
       // least window centre of its on-frame stamps
       {
@@ -349,7 +335,7 @@ __global__ void __launch_bounds__(kPThreads, 4) k_render_poly(const MixedArgs a)
                   for (int c = 0; c < NX; c += 2) {
                     const float2 v = make_float2(acc[r][c], c + 1 < NX ? acc[r][c + 1] : 0.f);
                     int2 hw, lw;
-                    if (decltype(fast)::value) deposit_split2(v, sc, sc_hi, hw, lw);
+                    if (decltype(fast)::value) fixed_split2_small(v, sc, sc_hi, hw, lw);
                     else fixed_split2_s(v, sc, sc_hi, hw, lw);
 #pragma unroll
                     for (int h = 0; h < 2 && c + h < NX; ++h) {
