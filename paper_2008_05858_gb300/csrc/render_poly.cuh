@@ -16,7 +16,12 @@
 // Measured on the 9216^2 frame of 340 slices x 6000 x 64 stamps: 3.4 ms (the edge tails 5.1 ms),
 // 4096^2 frame of 40 x 4000 x 32 0.21 ms (0.31).  Per stamp ~18 warp-instructions; the shared-
 // memory pipe is busy 60 % of the time, the FMA pipe 45 %, issue slots 60 %; four CTAs of 128
-// threads per SM (128 registers) leave the rest to latency.  Five CTAs spill (5.8 ms).
+// threads per SM (128 registers) leave the rest to latency.  Five CTAs spill (5.8 ms).  Windows of 9,
+// 13 and 15 px spill at four already (32 to 96 bytes a thread; the wide ones hold four pixel pairs'
+// coefficients and a tile quadrant of 7 x 7 pixels) and run three to an SM, with up to 168
+// registers: on the 4096^2 frame
+// K = 13 451 -> 377 us, K = 15 1237 -> 1178, K = 9 199 -> 190; 2473^2 frame of 40 x 3989 x 59 stamps,
+// K = 13, 768 -> 560 us (the edge tails 686).
 #pragma once
 #include <type_traits>
 
@@ -72,8 +77,11 @@ __host__ __device__ constexpr int quad_span(int R) { return (R + 1) / 2; }
 
 // CHECK: debug build of the same kernel, counting into a.err every deposit the plan did not
 // foresee.
+// CTAs per SM that a window's registers allow (above).
+__host__ __device__ constexpr int poly_ctas(int K) { return K >= 13 || K == 9 ? 3 : 4; }
+
 template <int K, int DX, int DY, bool CHECK>
-__global__ void __launch_bounds__(kPThreads, 4) k_render_poly(const MixedArgs a) {
+__global__ void __launch_bounds__(kPThreads, poly_ctas(K)) k_render_poly(const MixedArgs a) {
   constexpr int RX = K + DX, RY = K + DY, H = K / 2;
   constexpr int NS = poly_slots(K), F4 = poly_role_f4(K);
   constexpr int NX = quad_span(RX), NY = quad_span(RY);  // lane quadrant: columns and rows
