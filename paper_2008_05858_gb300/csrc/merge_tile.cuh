@@ -1,8 +1,8 @@
 // The tile merge of the tiled renderers: the boxes of the items overlapping one 64x32 output
 // tile are added per pixel in item order with compensated summation (TwoSum on the FP32
 // pairs, Neumaier's correction carried in a second word), converted and written once.  One
-// device function serves the standalone merge kernel (256 threads per tile) and the fused
-// merge at the end of the separable render kernel (128 threads), so both give the same bits.
+// device function serves the standalone merge kernel and the fused merge at the end of the
+// edge-tail render kernel (k_render_mixed), so both give the same bits.
 //
 // Fused merge: every tile counts its finished items.  A render CTA, after writing its box,
 // fences, adds one to the count of each tile the box overlaps, and the CTA that brings a

@@ -1,4 +1,5 @@
-// Mixed-precision tiled renderer (separable Gaussian PSF), its planner and the tile merge kernel.
+// Mixed-precision tiled renderer (separable Gaussian PSF, edge tails), its planner and the tile merge
+// kernel.
 //
 // Work item = one order-slice x a block of wavelength samples x a block of slit points.
 // Inside the item, a quad of lanes owns a *run* of B consecutive slit points of one wavelength
