@@ -492,13 +492,13 @@ def run_gpu(args):
         "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": headline_config(w, K, stamps, world, band),
         "precision": ("mixed (FP64 per-sample mapping coefficients, double-float FP32 mapping in s; "
-                      "FP32 stamps from double-float edge arguments; FP32 run sums of <= 16 stamps; "
+                      "FP32 stamps from per-sample polynomials in the sub-pixel offset; FP32 run sums of <= 16 stamps; "
                       "exact 52-bit fixed-point item boxes; TwoSum merge of FP32 pairs)"),
         "plan": plan,
         "roofline": roof, "roofline_other_pipe": other,
         "fp64_renderer": {"value": fp64_value, "unit": UNIT, "ms_per_step": statistics.median(fp64_ms),
                           "speedup_mixed_over_fp64": statistics.median(fp64_ms) / ms_per_step},
-        "kernel_ms": {"render_mixed (with the fused tile merge and the zero tiles)": kr, "merge_zero_tiles": km},
+        "kernel_ms": {"render_mixed (with the tile merge and the zero tiles)": kr, "merge_zero_tiles": km},
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                 "ms_per_step": statistics.median(e2e_ms), "steps": n_e2e,
                 "note": "spectra upload + render into pinned host memory + unload per step, the next step's "
@@ -952,7 +952,9 @@ def _load_spectrum_ptr(B, ctx, fiber, orders, lens, flux_tensor):
     return sid.value
 
 
-KERNEL_SOURCES = ["paper_2008_05858_gb300/csrc/render_mixed.cu", "paper_2008_05858_gb300/csrc/render_mixed_far.cu",
+KERNEL_SOURCES = ["paper_2008_05858_gb300/csrc/render_poly.cuh", "paper_2008_05858_gb300/csrc/render_poly.cu",
+                  "paper_2008_05858_gb300/csrc/poly_tables.cuh", "paper_2008_05858_gb300/csrc/fast_map.cuh",
+                  "paper_2008_05858_gb300/csrc/render_mixed.cu", "paper_2008_05858_gb300/csrc/render_mixed_far.cu",
                   "paper_2008_05858_gb300/csrc/render_mixed.cuh",
                   "paper_2008_05858_gb300/csrc/phi32.cuh",
                   "paper_2008_05858_gb300/csrc/mixed_common.cuh", "paper_2008_05858_gb300/csrc/merge_tile.cuh",
