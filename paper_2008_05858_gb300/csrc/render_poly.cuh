@@ -14,8 +14,8 @@
 // others hold the SM cost more (0.5 ms of a 9216^2 frame) than the separate launch (0.3 ms).
 //
 // Measured on the 9216^2 frame of 340 slices x 6000 x 64 stamps: 3.4 ms (the edge tails 5.1 ms),
-// 4096^2 frame of 40 x 4000 x 32 0.21 ms (0.31).  Per stamp ~18 warp-instructions; the shared-
-// memory pipe is busy 60 % of the time, the FMA pipe 45 %, issue slots 60 %; four CTAs of 128
+// 4096^2 frame of 40 x 4000 x 32 0.21 ms (0.31).  Per stamp ~20 warp-instructions; the shared-
+// memory pipe is busy 78 % of the time, the FMA pipe 44 %, issue slots 60 %; four CTAs of 128
 // threads per SM (128 registers) leave the rest to latency.  Five CTAs spill (5.8 ms).  Windows of 9,
 // 13 and 15 px spill at four already (32 to 96 bytes a thread; the wide ones hold four pixel pairs'
 // coefficients and a tile quadrant of 7 x 7 pixels) and run three to an SM, with up to 168
