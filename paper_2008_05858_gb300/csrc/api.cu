@@ -575,20 +575,30 @@ int plan_bands_and_tiles(Model* m) {
 }
 
 // Wavelength samples between two nodes of an elliptical slice's table (a multiple of 32), or 0
-// when its widths vary too fast or are too narrow: the cubic's error is 9/384 h^4 of the fourth
-// derivative in lt, and a pixel four widths from the centre changes at the rate 16 sigma'/sigma.
+// when its widths vary too fast or are too narrow.  The cubic through four nodes h apart errs by
+// 9/384 h^4 of the fourth derivative in lt.  A pixel r from the centre is exp(u) with
+// u = -r^2 / 2 sigma^2 to within its slower factors; four widths out, with p = |sigma' / sigma| and
+// q = |sigma'' / sigma|, that derivative is at most u1^4 + 6 u1^2 u2 + 4 u1 u3 + 3 u2^2 + u4 of the
+// pixel (u1 .. u4 below).  The curvature's terms do not fall with p: widths that hardly change need
+// them most.  The nodes reach two intervals beyond the slice's ends, and so do the bounds.
 int ellip_span(const e2e_order_slice& s) {
   if (!ellip_moments_supported(s.K)) return 0;
-  const int n_jb = (s.n_lambda + 31) / 32;
-  double rate = 0.0;
-  for (const double* c : {s.sigma_x, s.sigma_y}) {
-    const double lo = quad_min(c);
-    if (lo < kEllMinSigma) return 0;
-    rate = std::max(rate, 16.0 * (std::fabs(c[1]) + 2.0 * std::fabs(c[2])) / lo);
+  if (std::min(quad_min(s.sigma_x), quad_min(s.sigma_y)) < kEllMinSigma) return 0;
+  for (int g = (s.n_lambda + 31) / 32; g >= 1; g = std::min(g - 1, g * 7 / 8)) {
+    const double h = 64.0 * g / s.n_lambda, X = 1.0 + 2.0 * h;
+    double d4 = 0.0;
+    for (const double* c : {s.sigma_x, s.sigma_y}) {
+      const double over[3] = {c[0], c[1] * X, c[2] * X * X};  // the widths on [-X, X]
+      const double lo = quad_min(over);
+      if (lo < 0.5 * kEllMinSigma) d4 = HUGE_VAL;
+      const double p = (std::fabs(c[1]) + 2.0 * std::fabs(c[2]) * X) / lo, q = 2.0 * std::fabs(c[2]) / lo, p2 = p * p;
+      const double u1 = 16.0 * p, u2 = 48.0 * p2 + 16.0 * q, u3 = 192.0 * p2 * p + 144.0 * p * q;
+      const double u4 = 960.0 * p2 * p2 + 1152.0 * p2 * q + 144.0 * q * q;
+      d4 = std::max(d4, u1 * u1 * (u1 * u1 + 6.0 * u2) + 4.0 * u1 * u3 + 3.0 * u2 * u2 + u4);
+    }
+    if (9.0 / 384.0 * h * h * h * h * d4 <= kEllInterp) return 32 * g;
   }
-  const double h = 0.0455;  // (1e-7 * 384 / 9)^(1/4)
-  const double g = rate > 0.0 ? h / rate * s.n_lambda / 64.0 : (double)n_jb;
-  return g < 1.0 ? 0 : 32 * (int)std::min(g, (double)n_jb);
+  return 0;
 }
 
 // Node tables of an elliptical model, rebuilt on the device whenever its widths change; without
@@ -1095,7 +1105,7 @@ int render_impl(e2e_ctx* ctx, Model* m, int n_spec, const uint64_t* spec_ids, in
     }
   } else {
     for (auto& g : P.groups) {
-      KernelTimer kt(ctx, st, tab ? "render_table" : ellip ? "render_ellip" : "render_mixed");
+      KernelTimer kt(ctx, st, tab ? "render_table" : P.emom ? "render_moments" : ellip ? "render_ellip" : "render_mixed");
       E2E_CK(launch_items(ctx, m, g.K, g.first, g.count, d_table, store, st));
     }
     KernelTimer kt(ctx, st, "merge");

@@ -13,10 +13,10 @@
 //
 // C varies with the wavelength only through the widths.  It is tabulated at nodes along the slice
 // (every `span` samples, one more beyond either end) and interpolated by the cubic through four
-// nodes; the plan takes the span from the widths' rate of change so that the interpolation stays
-// below 1e-7 of a pixel four widths from the centre (and far below for brighter ones).  Truncated
-// at degree 10 the series is below 4e-8 of I + 1e-4 I(0) at widths 1.2 px, 3e-7 at 1.0 px (the
-// window's corners; 1e-9 of the peak).
+// nodes; the plan takes the span from the widths' slope and curvature so that the interpolation errs
+// by less than kEllInterp of a pixel four widths from the centre (and far less of brighter ones).
+// Truncated at degree 10 the series is below 4e-8 of I + 1e-4 I(0) at widths 1.2 px, 3e-7 at 1.0 px
+// (the window's corners; 1e-9 of the peak).
 #pragma once
 #include "e2e_device.cuh"
 
@@ -27,6 +27,7 @@ constexpr int kEllTerms = (kEllDegree + 1) * (kEllDegree + 2) / 2;          // 6
 constexpr int kEllEven = (kEllDegree / 2 + 1) * (kEllDegree / 2 + 1);       // 36: degrees 0, 2, .. 10
 constexpr int kEllRuns = 12;                                                // runs a warp turns into pixels at once
 constexpr double kEllMinSigma = 1.0;                                        // narrowest PSF the degree serves (px)
+constexpr double kEllInterp = 2e-7;                                         // interpolation error, four widths out
 constexpr int kEllMaxSlit = 128;                                            // slit points per item
 
 // Pixel pairs of a K x K window (the centre pairs with itself), and per lane of a warp.
