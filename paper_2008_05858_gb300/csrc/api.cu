@@ -479,6 +479,41 @@ int build_psf_tables(Model* m) {
   return rc;
 }
 
+// The photon renderer's FP32 copy of the slices' coefficients (photon.cu), at load and whenever
+// they change.
+int upload_photon_coefs(Model* m) {
+  const size_t nf = photon_coef_floats();
+  std::vector<float> cf(nf * m->slices.size(), 0.f);
+  for (size_t i = 0; i < m->slices.size(); ++i) {
+    const DevSlice& v = m->dev[i];
+    for (int c = 0; c < 2; ++c) {
+      const double* co = c ? v.cy : v.cx;
+      float* o = cf.data() + i * nf + c * kPhotonCoord;
+      double qb = 0.0, sb = 0.0;
+      for (int a = 0; a <= v.degree; ++a)
+        for (int b = 0; a + b <= v.degree; ++b) {
+          const int t = a + b, idx = t * (t + 1) / 2 + b;
+          o[idx] = (float)co[idx];
+          if (b == 0) qb += a * std::fabs(co[idx]);
+          else sb += std::fabs(co[idx]);
+        }
+      o[E2E_MAXC] = (float)qb;
+      o[E2E_MAXC + 1] = (float)sb;
+    }
+    float* e = cf.data() + i * nf + 2 * kPhotonCoord;  // sigma_x, sigma_y, slit-weight total
+    for (int k = 0; k < 3; ++k) {
+      e[k] = (float)v.sx[k];
+      e[3 + k] = (float)v.sy[k];
+    }
+    double total = 0.0;  // summed in order, as the running sums are
+    for (int k = 0; k < v.n_slit; ++k) total = k == 0 ? m->slices[i].u[k] : total + m->slices[i].u[k];
+    e[6] = (float)total;
+  }
+  if (!m->d_cf32) return upload(&m->d_cf32, cf.data(), cf.size());
+  if (!cf.empty()) E2E_CK(cudaMemcpy(m->d_cf32, cf.data(), cf.size() * sizeof(float), cudaMemcpyHostToDevice));
+  return E2E_OK;
+}
+
 // Bands and merge tiles of a planned model (every model, including one without slices, whose
 // tiles are all empty and merge to zeros).
 int plan_bands_and_tiles(Model* m) {
@@ -1532,36 +1567,11 @@ int e2e_load_model(e2e_ctx* ctx, const e2e_model_desc* desc_in, uint64_t* model_
   if (rc == E2E_OK) rc = upload(&m->d_u, u_all.data(), u_all.size());
   if (rc == E2E_OK) rc = upload(&m->d_ucum, ucum.data(), ucum.size());
   if (rc == E2E_OK) rc = upload(&m->d_usum, usum.data(), usum.size());
-  {
+  if (rc == E2E_OK) {
     std::vector<float> ucum32(ucum.begin(), ucum.end());
-    const size_t nf = photon_coef_floats();
-    std::vector<float> cf(nf * m->slices.size(), 0.f);
-    for (size_t i = 0; i < m->slices.size(); ++i) {
-      const DevSlice& v = ds[i];
-      for (int c = 0; c < 2; ++c) {
-        const double* co = c ? v.cy : v.cx;
-        float* o = cf.data() + i * nf + c * kPhotonCoord;
-        double qb = 0.0, sb = 0.0;
-        for (int a = 0; a <= v.degree; ++a)
-          for (int b = 0; a + b <= v.degree; ++b) {
-            const int t = a + b, idx = t * (t + 1) / 2 + b;
-            o[idx] = (float)co[idx];
-            if (b == 0) qb += a * std::fabs(co[idx]);
-            else sb += std::fabs(co[idx]);
-          }
-        o[E2E_MAXC] = (float)qb;
-        o[E2E_MAXC + 1] = (float)sb;
-      }
-      float* e = cf.data() + i * nf + 2 * kPhotonCoord;  // sigma_x, sigma_y, slit-weight total
-      for (int k = 0; k < 3; ++k) {
-        e[k] = (float)v.sx[k];
-        e[3 + k] = (float)v.sy[k];
-      }
-      e[6] = (float)usum[i];
-    }
-    if (rc == E2E_OK) rc = upload(&m->d_ucum32, ucum32.data(), ucum32.size());
-    if (rc == E2E_OK) rc = upload(&m->d_cf32, cf.data(), cf.size());
+    rc = upload(&m->d_ucum32, ucum32.data(), ucum32.size());
   }
+  if (rc == E2E_OK) rc = upload_photon_coefs(m.get());
   if (rc == E2E_OK) rc = upload(&m->d_bin_off, bin_off.data(), bin_off.size());
   if (rc == E2E_OK && m->psf == E2E_PSF_TABLE) rc = build_psf_tables(m.get());
   if (rc == E2E_OK) rc = upload(&m->d_dims, dims.data(), dims.size());
@@ -2052,6 +2062,7 @@ int e2e_update_model(e2e_ctx* ctx, uint64_t model_id, const double* cx_in, const
   }
   m->dev = dv;
   free_plan(m->plan);
+  if (int rc = upload_photon_coefs(m); rc != E2E_OK) return rc;
   return plan_model(m);
 }
 
