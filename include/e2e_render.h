@@ -174,8 +174,8 @@ const char* e2e_last_error(void);
  * model: the slices, the plan (items, merge tiles and their lists), and per wavelength sample
  * of every slice (degree + 3) x 16 bytes of precomputed mapping coefficients and PSF constants
  * (261 MB for a 9216^2 frame of 340 slices x 6000 samples at degree 5); a separable model whose
- * widths stay >= 1 px and windows K >= 3 adds its pixel-integral polynomials, 512 bytes per sample
- * at K = 11 (1.04 GB for that frame; left out where the device has no room for them); an
+ * widths stay >= 1 px and windows K >= 3 adds its pixel-integral polynomials, 448 bytes per sample
+ * at K = 11 (0.91 GB for that frame; left out where the device has no room for them); an
  * elliptical model whose widths stay >= 1 px and vary slowly from sample to sample adds the
  * pixel integrals' coefficients at nodes along the slices (25 KB per node at K = 13, a node per
  * hundred samples or so); the tabulated PSF adds its coefficient tables.

@@ -4,14 +4,17 @@
 // One thread per (slice, sample, axis).  The Gaussian at the pixel edges and centres is formed
 // in FP64 from one exponential (exp(-m^2 / 8 sigma^2) by a product recurrence: two
 // multiplications per half pixel), because its error would scale every coefficient; the Hermite
-// recurrences, their differences and the Chebyshev truncation run in FP32, where they add a few
-// 1e-8: the table of a 2.04e6-sample model costs ~0.2 ms instead of ~10 ms all in FP64.
+// recurrences and their differences (pixels near the centre), the Gauss-Legendre sums (wing
+// pixels) and the Chebyshev truncation run in FP32, where they add a few 1e-8: the table of a
+// 2.04e6-sample model costs a fraction of a millisecond instead of ~10 ms all in FP64.
 #include "e2e_kernels.h"
 #include "poly_tables.cuh"
+#include "quad_coeffs.h"
 
 namespace e2e {
 
 constexpr int kTaylorMax = 17;
+constexpr int kWingTaylor = 12;
 
 // Chebyshev truncation on |f| <= 1/2: f^n (n = 10..17) ~= sum over j = n mod 2, +2, ... <= 9 of
 // kChebCut[n - 10][j / 2] f^j (the expansion of f^n in T_k(2f), cut after k = 9; exact dyadic
@@ -41,6 +44,41 @@ __device__ __forceinline__ void hermite_edge(float phi, float xa2, float a2, flo
   }
 }
 
+// T(f) = G(i + f) e^(i f a + delta f) / phi(i) of a wing pixel (poly_tables.cuh), a = 1 / sigma^2 and
+// delta the rounding of the kernel's slope, less the leading term s0 = S(i):
+//
+//   T = e^(-f^2 a / 2 + delta f) S(i + f),   S(x) = int cosh(x a t) e^(-a t^2 / 2) dt over the pixel.
+//
+// S's Taylor coefficients are Gauss-Legendre sums of positive terms, so FP32 serves them.
+__device__ __forceinline__ void wing_taylor(int i, float a, float s0, float delta, float (&D)[kWingTaylor + 1]) {
+#pragma unroll
+  for (int n = 1; n <= kWingTaylor; ++n) D[n] = 0.f;
+  D[0] = s0;
+#pragma unroll 1
+  for (int q = kGl12 / 2; q < kGl12; ++q) {
+    const float t = (float)kGl12T[q], b = a * t, e = expf((float)i * b);
+    float p = (float)kGl12W[q] * expf(-0.5f * b * t);  // two nodes' weight, half a cosh each
+    const float ch = e + 1.f / e, sh = e - 1.f / e;
+#pragma unroll
+    for (int n = 1; n <= kWingTaylor; ++n) {
+      p *= b * (1.f / (float)n);
+      D[n] = fmaf(p, (n & 1) ? sh : ch, D[n]);
+    }
+  }
+  const float h = -0.5f * a;
+#pragma unroll
+  for (int n = kWingTaylor; n >= 2; --n) {  // times e^(h f^2)
+    float c = 1.f;
+#pragma unroll
+    for (int k = 1; 2 * k <= n; ++k) {
+      c *= h * (1.f / (float)k);
+      D[n] = fmaf(c, D[n - 2 * k], D[n]);
+    }
+  }
+#pragma unroll
+  for (int n = kWingTaylor; n >= 1; --n) D[n] = fmaf(delta, D[n - 1], D[n]);
+}
+
 __global__ void __launch_bounds__(128) k_poly_tables(const DevSlice* __restrict__ slices) {
   const DevSlice& S = slices[blockIdx.y];
   const int K = S.K, H = K / 2;
@@ -57,12 +95,14 @@ __global__ void __launch_bounds__(128) k_poly_tables(const DevSlice* __restrict_
     double w = exp(-0.125 * a * a);
     const double r = w * w;
     const float a2 = (float)(a * a);
+    const float4 ge = S.samples[(int64_t)j * (S.degree + 3) + S.degree + 1];
+    const float gk = axis ? ge.z : ge.x;  // the kernel's slope constant
     float lo[kTaylorMax], hi[kTaylorMax];  // edges i - 1/2 and i + 1/2
     for (int i = 0; i <= H; ++i) {
       const double gc = g;  // the pixel's centre, m = 2i
       g *= w;
       w *= r;
-      hermite_edge((float)g, (float)((i + 0.5) * a * a), a2, hi);
+      if (i < kPolyWing) hermite_edge((float)g, (float)((i + 0.5) * a * a), a2, hi);
       g *= w;
       w *= r;
       if (i == 0) {  // the centre pixel's left edge is the mirror image of its right one
@@ -87,31 +127,64 @@ __global__ void __launch_bounds__(128) k_poly_tables(const DevSlice* __restrict_
         }
       }
       const double c0 = gc * (1.0 + (double)s);
-      // Taylor coefficients of G(i + f) and their truncation to degree kPolyDegree
+      const int m = H - i, half = m & 1, slot = m >> 1, terms = poly_terms(K, slot);
       float E[kPolyTerms], O[kPolyTerms];
 #pragma unroll
       for (int q = 0; q < kPolyTerms; ++q) E[q] = O[q] = 0.f;
+      if (i < kPolyWing) {
+        // Taylor coefficients of G(i + f) and their truncation to degree kPolyDegree
 #pragma unroll
-      for (int d = kTaylorMax; d >= 1; --d) {
-        const float v = (hi[d - 1] - lo[d - 1]) * ((d & 1) ? 1.f / (float)d : -1.f / (float)d);
-        if (d > kPolyDegree) {
+        for (int d = kTaylorMax; d >= 1; --d) {
+          const float v = (hi[d - 1] - lo[d - 1]) * ((d & 1) ? 1.f / (float)d : -1.f / (float)d);
+          if (d > kPolyDegree) {
 #pragma unroll
-          for (int q = 0; q < kPolyTerms; ++q) {
-            if (d & 1) O[q] = fmaf(v, kChebCut[d - 10][q], O[q]);
-            else E[q] = fmaf(v, kChebCut[d - 10][q], E[q]);
+            for (int q = 0; q < kPolyTerms; ++q) {
+              if (d & 1) O[q] = fmaf(v, kChebCut[d - 10][q], O[q]);
+              else E[q] = fmaf(v, kChebCut[d - 10][q], E[q]);
+            }
+          } else if (d & 1) {
+            O[d / 2] += v;
+          } else {
+            E[d / 2] += v;
           }
-        } else if (d & 1) {
-          O[d / 2] += v;
-        } else {
-          E[d / 2] += v;
+        }
+      } else {
+        float D[kWingTaylor + 1];
+        const double slope = 0.69314718055994530942 * (double)poly_wing_rate(gk, i) - (double)i * a * a;
+        wing_taylor(i, a2, 1.f + s, (float)slope, D);
+        const float gf = (float)gc;
+#pragma unroll
+        for (int d = kWingTaylor; d >= 1; --d) {
+          const float v = gf * D[d];
+          if (d > kPolyDegree) {
+#pragma unroll
+            for (int q = 0; q < kPolyTerms; ++q) {
+              if (d & 1) O[q] = fmaf(v, kChebCut[d - 10][q], O[q]);
+              else E[q] = fmaf(v, kChebCut[d - 10][q], E[q]);
+            }
+          } else if (d & 1) {
+            O[d / 2] += v;
+          } else {
+            E[d / 2] += v;
+          }
+        }
+        if (terms < kPolyTerms) {  // f^8 and f^9 in their turn, cut to degree 7
+          static_assert(kPolyTerms == 5, "the cuts below");
+          constexpr float ce[4] = {-3.0517578125e-05f, 0.00390625f, -0.078125f, 0.5f};
+          constexpr float co[4] = {-0.0001373291015625f, 0.00732421875f, -0.10546875f, 0.5625f};
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            E[q] = fmaf(E[4], ce[q], E[q]);
+            O[q] = fmaf(O[4], co[q], O[q]);
+          }
         }
       }
       E[0] = (float)(c0 + (double)E[0]);
-      const int m = H - i, half = m & 1, slot = m >> 1;
       float2* out = reinterpret_cast<float2*>(const_cast<float4*>(S.poly) + ((int64_t)j * 4 + 2 * half + axis) * f4) +
-                    slot * kPolyTerms;
+                    poly_at(K, slot);
 #pragma unroll
-      for (int q = 0; q < kPolyTerms; ++q) out[q] = make_float2(E[q], i == 0 ? 0.f : O[q]);
+      for (int q = 0; q < kPolyTerms; ++q)
+        if (q < terms) out[q] = make_float2(E[q], i == 0 ? 0.f : O[q]);
 #pragma unroll
       for (int k = 0; k < kTaylorMax; ++k) lo[k] = hi[k];
     }

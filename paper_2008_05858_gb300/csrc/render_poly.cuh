@@ -8,7 +8,9 @@
 // depend on the wavelength sample only.  A warp takes eight samples, a quad of lanes each, and
 // walks all the item's slit points with them, so that a lane loads its coefficients once per
 // sample and holds them in registers: lane (axis, half) of the quad evaluates half the pixel pairs
-// of one axis of every stamp, 12 packed and 12 scalar operations per stamp at K = 11.  The quad's
+// of one axis of every stamp, at K = 11 some two dozen packed and scalar operations and, for the
+// slopes of its two wing pairs, four exponentials (3 % of the 9216^2 frame below, 3.79 -> 3.91 ms
+// with its merge; without them narrow PSFs' wings miss the bound, poly_tables.cuh).  The quad's
 // profiles go through shared memory, and each lane adds one quadrant of the tile's outer product.
 // The tiles are merged by a kernel of their own: the last CTA of a tile merging it while three
 // others hold the SM cost more (0.5 ms of a 9216^2 frame) than the separate launch (0.3 ms).
@@ -29,6 +31,7 @@
 #include "e2e_kernels.h"
 #include "fast_map.cuh"
 #include "mixed_common.cuh"
+#include "phi32.cuh"
 #include "poly_tables.cuh"
 
 namespace e2e {
@@ -187,13 +190,22 @@ __global__ void __launch_bounds__(kPThreads, poly_ctas(K)) k_render_poly(const M
 #pragma unroll
     for (int s = 0; s < NS; ++s)
 #pragma unroll
-      for (int q = 0; q < kPolyTerms; ++q) {
-        const int e = s * kPolyTerms + q;
+      for (int q = 0; q < poly_terms(K, s); ++q) {
+        const int e = poly_at(K, s) + q;
         cf[s][q] = (e & 1) ? make_float2(cv[e / 2].z, cv[e / 2].w) : make_float2(cv[e / 2].x, cv[e / 2].y);
       }
     const float2 wj = jvalid ? tabW[jc] : make_float2(0.f, 0.f);
     const float4* Pj = tabP + jc * (nd + 2);
     const FastMap fm(Pj, S.degree);
+    float wing[NS];  // slopes of this lane's wing pixels (the other pixel of such a slot has none)
+    {
+      const float4 ge = Pj[nd];
+#pragma unroll
+      for (int s = 0; s < NS; ++s) {
+        const int i = H - half - 2 * s;
+        wing[s] = i >= kPolyWing ? poly_wing_rate(axis ? ge.z : ge.x, i) : 0.f;
+      }
+    }
     int parity = 0;
     for (int k0 = 0; k0 < it.nk; k0 += 16) {
       const int nk = min(16, it.nk - k0);
@@ -279,23 +291,32 @@ __global__ void __launch_bounds__(kPThreads, poly_ctas(K)) k_render_poly(const M
               z[e] = f * f;
               fw[e] = f * mult[e];
 #pragma unroll
-              for (int s = 0; s < NS; ++s) p[e][s] = cf[s][kPolyTerms - 1];
+              for (int s = 0; s < NS; ++s) p[e][s] = cf[s][poly_terms(K, s) - 1];
             }
 #pragma unroll
             for (int q = kPolyTerms - 2; q >= 0; --q)
 #pragma unroll
               for (int e = 0; e < 2; ++e)
 #pragma unroll
-                for (int s = 0; s < NS; ++s) p[e][s] = __ffma2_rn(p[e][s], make_float2(z[e], z[e]), cf[s][q]);
+                for (int s = 0; s < NS; ++s)
+                  if (q < poly_terms(K, s) - 1) p[e][s] = __ffma2_rn(p[e][s], make_float2(z[e], z[e]), cf[s][q]);
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
               float* row = wrow + (parity + e) * kPBuf;
 #pragma unroll
               for (int s = 0; s < NS; ++s) {
-                const float Ew = p[e][s].x * mult[e];
+                float2 v;  // G(i + f), G(i - f)
+                if (poly_wing(K, s)) {
+                  const float f = axis ? st[e].y : st[e].x, t = f * wing[s];
+                  v = __ffma2_rn(make_float2(p[e][s].y, p[e][s].y), make_float2(f, -f), make_float2(p[e][s].x, p[e][s].x));
+                  v = __fmul2_rn(v, __fmul2_rn(make_float2(mult[e], mult[e]), make_float2(ex2_approx(-t), ex2_approx(t))));
+                } else {
+                  const float Ew = p[e][s].x * mult[e];
+                  v = make_float2(fmaf(fw[e], p[e][s].y, Ew), fmaf(-fw[e], p[e][s].y, Ew));
+                }
                 if (2 * s + 1 <= H || half == 0) {  // half 1 has one pair fewer when H is even
-                  row[2 * s] = fmaf(fw[e], p[e][s].y, Ew);
-                  row[K - 1 - 2 * half - 2 * s] = fmaf(-fw[e], p[e][s].y, Ew);
+                  row[2 * s] = v.x;
+                  row[K - 1 - 2 * half - 2 * s] = v.y;
                 }
               }
             }
