@@ -57,7 +57,9 @@ enum { E2E_PSF_SEPARABLE = 0, E2E_PSF_ELLIPTICAL = 1, E2E_PSF_TABLE = 2 };
  *                 those of that mapping, the offset in the pixel may be rounded to ~1e-7 px);
  *                 FP32 PSF stamps, from polynomials in that offset where a separable model's
  *                 widths stay >= 1 px, else from double-float edge arguments; FP32 sums
- *                 over runs of <= 16 stamps in registers; each item's box summed exactly in
+ *                 over runs of <= 16 stamps in registers (elliptical PSFs >= 1.3 px wide: 66
+ *                 moments of a run of <= 128 stamps, the moments and the large terms of the
+ *                 pixels summed with their rounding errors); each item's box summed exactly in
  *                 52-bit fixed point (shared-memory integer atomics) and stored as an FP32
  *                 (hi, lo) pair; boxes merged into the frame with TwoSum compensation (the
  *                 fast path: per-pixel error <= 1e-6 relative against the FP64 definition).
@@ -176,8 +178,8 @@ const char* e2e_last_error(void);
  * (261 MB for a 9216^2 frame of 340 slices x 6000 samples at degree 5); a separable model whose
  * widths stay >= 1 px and windows K >= 3 adds its pixel-integral polynomials, 448 bytes per sample
  * at K = 11 (0.91 GB for that frame; left out where the device has no room for them); an
- * elliptical model whose widths stay >= 1 px and vary slowly from sample to sample adds the
- * pixel integrals' coefficients at nodes along the slices (25 KB per node at K = 13, a node per
+ * elliptical model's slices whose widths stay >= 1.3 px and vary slowly from sample to sample add
+ * the pixel integrals' coefficients at nodes along them (25 KB per node at K = 13, a node per
  * hundred samples or so); the tabulated PSF adds its coefficient tables.
  * Errors: E2E_EINVAL, E2E_ENOMEM, E2E_ECUDA. */
 int e2e_load_model(e2e_ctx* ctx, const e2e_model_desc* desc, uint64_t* model_id);

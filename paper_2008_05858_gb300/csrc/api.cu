@@ -70,7 +70,9 @@ struct Plan {
   int B_adj = 1;      // run length of the adjoint (its FP32 sums run over one run)
   int poly = 0;       // separable kernel: polynomial pixel integrals (every sample's table is built)
   int tcap = 0, tcells = 0;  // tabulated PSF: stamps a CTA stages at a time; most phase cells of a slice
-  int emom = 0;       // elliptical: rendered on run moments (every slice's nodes are built)
+  int emom = 0;       // elliptical: the slices with node tables are rendered on run moments
+  int nk_mom = 1;     // ... most slit points of such an item, and its kernel's shared memory
+  size_t smem_mom = 0;
   std::vector<EllGroup> egroups;  // its CTAs' items, in item order
   EllGroup* d_egroups = nullptr;
   int far_tails = 0;  // separable kernel: every tail edge's argument within the cheaper rational's fit
@@ -85,6 +87,7 @@ struct Plan {
   // items grouped by K (one kernel launch per group)
   struct Group {
     int K, first, count;
+    bool mom;  // elliptical: items of the moments render
   };
   std::vector<Group> groups;
   // y-bands: within each K group the items are ordered by the band of their box's first row,
@@ -636,8 +639,8 @@ int ellip_span(const e2e_order_slice& s) {
   return 0;
 }
 
-// Node tables of an elliptical model, rebuilt on the device whenever its widths change; without
-// them (a slice's widths, or no room) the model renders stamp by stamp.
+// Node tables of an elliptical model, rebuilt on the device whenever its widths change, for the slices
+// that they serve; the others (or all, where there is no room) render stamp by stamp.
 int build_ellip_nodes(Model* m) {
   m->plan.emom = 0;
   const int ns = (int)m->slices.size();
@@ -647,23 +650,24 @@ int build_ellip_nodes(Model* m) {
   m->d_enodes = nullptr;
   int64_t total = 0;
   int max_nodes = 0;
-  std::vector<int64_t> off(ns);
+  std::vector<int64_t> off(ns, -1);
   for (int i = 0; i < ns; ++i) {
     const auto& s = m->slices[i].d;
     const int span = ellip_span(s);
-    if (!span) return E2E_OK;
+    if (!span) continue;
     m->dev[i].espan = span;
     const int n = (s.n_lambda + span - 1) / span + 3;
     max_nodes = std::max(max_nodes, n);
     off[i] = total;
     total += n * ellip_node_floats(s.K);
   }
+  if (total == 0) return E2E_OK;
   if (cudaMalloc((void**)&m->d_enodes, (size_t)total * sizeof(float)) != cudaSuccess) {
     cudaGetLastError();
     m->d_enodes = nullptr;
     return E2E_OK;
   }
-  for (int i = 0; i < ns; ++i) m->dev[i].enodes = m->d_enodes + off[i];
+  for (int i = 0; i < ns; ++i) m->dev[i].enodes = off[i] < 0 ? nullptr : m->d_enodes + off[i];
   E2E_CK(cudaMemcpy(m->d_slices, m->dev.data(), ns * sizeof(DevSlice), cudaMemcpyHostToDevice));
   E2E_CK(launch_ellip_nodes(m->d_slices, ns, max_nodes, 0));
   E2E_CK(cudaDeviceSynchronize());
@@ -820,17 +824,19 @@ int plan_model(Model* m) {
     P.items.clear();
     P.groups.clear();
     P.JB = 1;
-    for (int Kg : m->Ks) {
-      Plan::Group g{Kg, (int)P.items.size(), 0};
+    for (size_t kg = 0; kg < m->Ks.size() * (P.emom ? 2 : 1); ++kg) {  // per K; with moments: stamps, then moments
+      const int Kg = m->Ks[P.emom ? kg / 2 : kg];
+      const bool mom = P.emom && kg % 2 == 1;
+      Plan::Group g{Kg, (int)P.items.size(), 0, mom};
       for (int i = 0; i < ns; ++i) {
         const auto& s = m->slices[i].d;
-        if (s.K != Kg) continue;
+        if (s.K != Kg || (P.emom && (m->dev[i].enodes != nullptr) != mom)) continue;
         const int nrc_full = (s.n_slit + P.B - 1) / P.B;
         int KC = nrc_full <= 16 ? n_k16[i] : P.B;  // 16-point blocks per item
         const int nrc = std::min(nrc_full, (KC * 16 + P.B - 1) / P.B);
         int JB = std::max(1, std::min(jb_cap, std::min((8 + nrc - 1) / nrc, 16 / nrc)));
         if (ellip) KC = JB = 1;  // <= 512 stamps: <= 512 deposits per box pixel
-        if (P.emom) {            // the slit in equal parts of at most kEllMaxSlit points
+        if (mom) {               // the slit in equal parts of at most kEllMaxSlit points
           const int parts = (n_k16[i] * 16 + kEllMaxSlit - 1) / kEllMaxSlit;
           KC = (n_k16[i] + parts - 1) / parts;
         }
@@ -866,29 +872,37 @@ int plan_model(Model* m) {
             g.count++;
           }
       }
-      P.groups.push_back(g);
+      if (g.count > 0 || !P.emom) P.groups.push_back(g);
     }
     P.store_elems = store;
     P.max_area = 0;
-    P.nk_max = 1;
-    for (auto& it : P.items) {
-      P.max_area = std::max(P.max_area, it.bw * it.bh);
-      P.nk_max = std::max(P.nk_max, it.nk);
+    P.nk_max = P.nk_mom = 1;
+    int area_mom = 0, area = 0, K_mom = 3;
+    for (const auto& g : P.groups) {
+      if (g.mom) K_mom = std::max(K_mom, g.K);
+      for (int n = g.first; n < g.first + g.count; ++n) {
+        const Item& it = P.items[n];
+        int& ar = g.mom ? area_mom : area;
+        int& nk = g.mom ? P.nk_mom : P.nk_max;
+        ar = std::max(ar, it.bw * it.bh);
+        nk = std::max(nk, it.nk);
+      }
     }
+    P.max_area = std::max(area, area_mom);
     for (auto& s : m->slices) {
       const int c = (int)s.d.map_oversample + (s.d.map_size % 2 == 0 ? 1 : 0);  // phase cells per axis
       if (m->psf == E2E_PSF_TABLE) P.tcells = std::max(P.tcells, c * c);
     }
-    P.smem = m->psf == E2E_PSF_TABLE ? table_smem_bytes(P.max_area, P.nk_max, P.max_deg + 1, P.tcells,
+    P.smem = m->psf == E2E_PSF_TABLE ? table_smem_bytes(area, P.nk_max, P.max_deg + 1, P.tcells,
                                                         (size_t)optin - kStaticSmemReserve, &P.tcap)
-             : P.emom ? ellip_moment_smem(m->Ks.back(), P.max_area, P.nk_max, P.max_deg + 1)
-             : ellip ? ellip_smem_bytes(P.max_area, P.nk_max, P.max_deg + 1, m->Ks.empty() ? 15 : m->Ks.front())
-             : P.poly ? poly_smem_bytes(P.max_area, P.JB, P.nk_max, P.max_deg + 1)
-                     : mixed_smem_bytes(P.max_area, P.JB, P.nk_max, P.B, P.max_deg + 1);
+             : ellip ? ellip_smem_bytes(area, P.nk_max, P.max_deg + 1, m->Ks.empty() ? 15 : m->Ks.front())
+             : P.poly ? poly_smem_bytes(area, P.JB, P.nk_max, P.max_deg + 1)
+                     : mixed_smem_bytes(area, P.JB, P.nk_max, P.B, P.max_deg + 1);
+    P.smem_mom = P.emom ? ellip_moment_smem(K_mom, area_mom, P.nk_mom, P.max_deg + 1) : 0;
     // the polynomial kernel's warps take eight samples each through the whole slit: a grid that
     // would not fill the GPU gets items of one 32-sample block (a sample octet per warp)
     const bool thin = P.poly && jb_cap > 1 && P.JB > 1 && (int)P.items.size() < kPolyWave;
-    if ((int)P.smem + kStaticSmemReserve <= optin && !thin) break;
+    if ((int)std::max(P.smem, P.smem_mom) + kStaticSmemReserve <= optin && !thin) break;
     if (jb_cap == 1 && !P.emom)
       return fail(E2E_EINVAL, "trace footprint of a work item exceeds on-chip memory (area " +
                                   std::to_string(P.max_area) + " px)");
@@ -899,7 +913,8 @@ int plan_model(Model* m) {
     // a CTA's items: neighbours of one slice, interval and band, at most four (each CTA loads its
     // interval's nodes once), fewer where the GPU would run out of CTAs
     const int cap = std::max(1, std::min(4, (int)P.items.size() / (152 * 4)));
-    for (size_t s = 0; s < P.seg_count.size(); ++s)
+    for (size_t s = 0; s < P.seg_count.size(); ++s) {
+      if (!P.groups[s / P.n_bands].mom) continue;
       for (int n = P.seg_first[s]; n < P.seg_first[s] + P.seg_count[s]; ++n) {
         const Item& it = P.items[n];
         const int v = it.j0 / m->dev[it.slice].espan;
@@ -908,6 +923,7 @@ int plan_model(Model* m) {
           P.egroups.push_back(EllGroup{n, 0, v, 0});
         P.egroups.back().count++;
       }
+    }
     return upload(&P.d_egroups, P.egroups.data(), P.egroups.size());
   }
   return E2E_OK;
@@ -1015,14 +1031,14 @@ cudaError_t launch_items(e2e_ctx* ctx, Model* m, int K, int first, int count, co
     return launch_render_table(K, m->d_slices, m->d_ts, m->d_T32, m->d_field, d_table, m->d_u,
                                P.d_items + first, count, store, P.nk_max, P.max_deg, P.tcap, P.tcells, P.smem, st,
                                ctx->d_err);
-  if (P.emom) {
+  if (P.emom && count > 0 && m->dev[P.items[first].slice].enodes) {
     auto at = [&](int n) {
       return std::lower_bound(P.egroups.begin(), P.egroups.end(), n,
                               [](const EllGroup& g, int i) { return g.first < i; }) - P.egroups.begin();
     };
     const int g0 = (int)at(first), g1 = (int)at(first + count);
     return launch_ellip_moments(K, m->d_slices, d_table, m->d_u, P.d_items, P.d_egroups + g0, g1 - g0, store,
-                                P.nk_max, P.max_deg, P.smem, st, ctx->d_err);
+                                P.nk_mom, P.max_deg, P.smem_mom, st, ctx->d_err);
   }
   if (m->psf == E2E_PSF_ELLIPTICAL)
     return launch_render_ellip(K, m->d_slices, d_table, m->d_u, P.d_items + first, count, store, P.nk_max,
@@ -1140,7 +1156,7 @@ int render_impl(e2e_ctx* ctx, Model* m, int n_spec, const uint64_t* spec_ids, in
     }
   } else {
     for (auto& g : P.groups) {
-      KernelTimer kt(ctx, st, tab ? "render_table" : P.emom ? "render_moments" : ellip ? "render_ellip" : "render_mixed");
+      KernelTimer kt(ctx, st, tab ? "render_table" : g.mom ? "render_moments" : ellip ? "render_ellip" : "render_mixed");
       E2E_CK(launch_items(ctx, m, g.K, g.first, g.count, d_table, store, st));
     }
     KernelTimer kt(ctx, st, "merge");

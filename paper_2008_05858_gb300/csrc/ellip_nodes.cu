@@ -48,6 +48,7 @@ __device__ __forceinline__ double between(double a, double b) {
 __global__ void __launch_bounds__(128) k_ellip_nodes(const DevSlice* __restrict__ slices) {
   constexpr int N = kEllTaylor;
   const DevSlice& S = slices[blockIdx.y];
+  if (!S.enodes) return;  // a slice that renders stamp by stamp
   const int n_int = (S.n_lambda + S.espan - 1) / S.espan;
   const int K = S.K, H = K / 2, NP = ell_pairs(K), NS = ell_slots(K) * 32;
   if ((int)blockIdx.x >= n_int + 3) return;

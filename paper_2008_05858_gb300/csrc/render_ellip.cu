@@ -1,6 +1,6 @@
 // Elliptical (rotated) Gaussian PSF: the plain FP64 renderer, and the mixed-precision tiled renderer
-// of the models that render_ellip_moments.cu does not take (K of 1 or 15, widths below 1 px or
-// changing fast along the slice; 3 x 4 x 2 traces of 8000 x 128 stamps, K = 13: 8.9 ms here, 2.5 there).
+// of the slices that render_ellip_moments.cu does not take (K of 1 or 15, widths below 1.3 px or
+// changing fast along the slice; 3 x 4 x 2 traces of 8000 x 128 stamps, K = 13: 8.9 ms here, 3.3 there).
 //
 // The PSF of an order-slice is a bivariate normal with widths sigma_a(lt), sigma_b(lt) along
 // axes rotated by theta (the asymmetric Gaussian of Sec. 2.2, with a rotation).  Its pixel

@@ -2,11 +2,10 @@
 //
 // k_render_ellip (render_ellip.cu) evaluates every stamp's K^2 pixel integrals: 253 warp-
 // instructions a stamp at K = 13.  Here a stamp adds its 66 moments to its run's, and a warp turns
-// the runs of a wavelength sample into pixels together: 57 warp-instructions a stamp at 128 slit
-// points of 8 px (a dozen stamps per run), a third of them the product of the sample's
-// coefficients with the runs' moments, in packed pairs of runs.
+// the runs of a wavelength sample into pixels together: some 75 warp-instructions a stamp at 128 slit
+// points of 8 px (a dozen stamps per run).
 //
-// One CTA of 16 warps takes the items of one slice between two nodes: their four node tables become
+// One CTA of 12 warps takes the items of one slice between two nodes: their four node tables become
 // the cubics' coefficients in shared memory (float4 per term and pixel pair, 101 KB at K = 13).  A
 // warp takes one sample and walks its slit points 32 at a time: each lane maps one stamp and forms
 // its Chebyshev values; the run boundaries are a ballot; 21 lanes hold the 66 moments as 2 x 2
@@ -14,10 +13,13 @@
 // pixels, lane l the pixel pairs l, l + 32, ..., and deposits them into the item's box as exact
 // fixed point (the low word 20 bits wide: an item may put 4096 deposits on a pixel).
 //
-// Measured on 24 slices x 8000 x 128 stamps (K = 13): 8.59 -> 2.3 ms, error against 64 bits 3.6e-8
-// -> 2.8e-8.  The shared-memory pipe is busy 65 % of the time (the coefficients, 12 wavefronts per
-// term and sample), issue slots 46 %; the tables leave room for one CTA per SM, so its prologue and
-// write-back (8 of 61 us per item) stand by themselves.
+// Measured on 24 slices x 8000 x 128 stamps (K = 13), the whole render: 8.85 ms stamp by stamp, 2.52
+// with every sum in plain FP32 (and the far wings of runs on one side of their pixel up to 3.5 times
+// the bound off), 3.33 with the errors of the large sums carried (ellip_moments.cuh): 0.2 ms for the
+// moments', 0.2 for the pixels', the rest because the sums of twelve runs and their errors take 168
+// registers, so 12 warps instead of 16 (at 16 they spill: 3.7 to 4.4 ms; slot by slot without a spill,
+// the moments read three times, 3.6).  Issue slots are busy half the time, the shared-memory pipe
+// half; one CTA per SM, so its prologue and write-back stand by themselves.
 #include "e2e_device.cuh"
 #include "e2e_kernels.h"
 #include "ellip_moments.cuh"
@@ -26,7 +28,7 @@
 
 namespace e2e {
 
-constexpr int kMThreads = 512;
+constexpr int kMThreads = 384;
 constexpr int kMWarps = kMThreads / 32;
 constexpr int kMStage = 16;  // stamps staged at a time
 // A staged pair of stamps: 12 float4 {v, v' of the first, v, v' of the second}, (v, v') the values
@@ -35,11 +37,12 @@ constexpr int kMStage = 16;  // stamps staged at a time
 constexpr int kMPair = 52;
 
 struct MomentLayout {
-  size_t tab, mom, stage, tabP, tabS, tabU, tabW, boxh, boxl, total;
+  size_t tab, mom, low, stage, tabP, tabS, tabU, tabW, boxh, boxl, total;
   __host__ __device__ MomentLayout(int slots, int NK, int nd, int area) {
     size_t o = 0;
     tab = o; o += (size_t)kEllTerms * slots * 32 * 16;           // cubic coefficients in the interval
     mom = o; o += (size_t)kMWarps * (kEllTerms + 1) * kEllRuns * 4;  // [term][run] moments per warp, a spare row
+    low = o; o += (size_t)kMWarps * (kEllLow + 1) * kEllRuns * 4;  // the low words of the first few
     stage = o; o += (size_t)kMWarps * kMStage / 2 * kMPair * 4;
     tabP = o; o += (size_t)32 * (nd + 2) * 16;                   // the item's rows of the sample table
     tabS = o; o += (size_t)NK * 8;
@@ -73,6 +76,9 @@ __device__ __forceinline__ float2 fixed20_to_pair(int hi, int lo, float scale) {
   return fixed_to_pair(hi >> 2, ((unsigned)(hi & 3) << 20) | (unsigned)lo, scale);
 }
 
+// a - b as one packed FMA (no negated copies).
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+
 struct MomentArgs {
   MixedArgs a;
   const EllGroup* groups;
@@ -91,6 +97,7 @@ __global__ void __launch_bounds__(kMThreads, 1) k_ellip_moments(const MomentArgs
   const MomentLayout L(SL, a.nk_max, a.max_deg + 1, 0);
   float4* tab = reinterpret_cast<float4*>(smem + L.tab);
   float* mom = reinterpret_cast<float*>(smem + L.mom) + warp * (kEllTerms + 1) * R;
+  float* low = reinterpret_cast<float*>(smem + L.low) + warp * (kEllLow + 1) * R;
   float* stage = reinterpret_cast<float*>(smem + L.stage) + warp * (kMStage / 2) * kMPair;
   float4* tabP = reinterpret_cast<float4*>(smem + L.tabP);
   float2* tabS = reinterpret_cast<float2*>(smem + L.tabS);
@@ -115,25 +122,19 @@ __global__ void __launch_bounds__(kMThreads, 1) k_ellip_moments(const MomentArgs
     pb -= 6 - pa;
     ++pa;
   }
-  // and where a run's go in mom (past the triangle: the spare row).  Two of the other lanes sum the
-  // weights themselves, M_00, from their leading 12 bits (exact) and the rest: a sum of a dozen
-  // FP32 weights would round M_00, and with it every pixel of the run, by 1e-7.
-  int mrow[4];
+  // and where a run's go in mom and low (past the triangle, or above degree 2: the spare rows).  Two
+  // of the other lanes sum the weights themselves, M_00, from their leading 12 bits and the rest,
+  // which holds what an FP32 weight leaves out.
+  int mrow = 0, lrow = 0;  // a row a byte
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int ta = 2 * pa + (q >> 1), tb = 2 * pb + (q & 1);
-    mrow[q] = (pa < 6 && ta + tb <= kEllDegree ? ell_term(ta, tb) : kEllTerms) * R;
+    const int term = pa < 6 && ta + tb <= kEllDegree ? ell_term(ta, tb) : kEllTerms;
+    mrow |= term << (8 * q);
+    lrow |= ell_low_row(term) << (8 * q);
   }
   const float* sx = stage + 4 * (pa < 6 ? pa : lane == 21 ? 5 : 6);
   const float* sy = stage + 4 * (pa < 6 ? 6 + pb : lane == 21 ? 6 : 11);
-  // the lane's pixels: offsets in the window of its pairs' first pixels
-  int pm[SL], pn[SL];
-#pragma unroll
-  for (int i = 0; i < SL; ++i) {
-    const int e = min(lane + 32 * i, NP - 1);
-    pn[i] = e / K;
-    pm[i] = e - pn[i] * K;
-  }
   const double* flux = a.flux_tab[S.flux_slot];
   const double* u = a.u_all + S.u_off;
   const double inv_ns = 1.0 / (double)S.n_slit;
@@ -181,9 +182,12 @@ __global__ void __launch_bounds__(kMThreads, 1) k_ellip_moments(const MomentArgs
     frexp(total, &ex);
     const int Psh = total > 0.0 ? max(-100, min(100, 52 - ex)) : 0;
     const float sc = ldexpf(1.f, Psh), sc_hi = ldexpf(1.f, Psh - 20);
-    int off[SL];  // the lane's pixels in the box, and the sum of a pair's
+    int off[SL];  // the first pixels of the lane's pairs, in the box from the window's origin
 #pragma unroll
-    for (int i = 0; i < SL; ++i) off[i] = pn[i] * it.bw + pm[i];
+    for (int i = 0; i < SL; ++i) {
+      const int e = min(lane + 32 * i, NP - 1);
+      off[i] = (e / K) * it.bw + e % K;
+    }
     const int last = (K - 1) * (it.bw + 1);
 
     for (int jj = warp; jj < it.nj && total > 0.0; jj += kMWarps) {
@@ -191,7 +195,8 @@ __global__ void __launch_bounds__(kMThreads, 1) k_ellip_moments(const MomentArgs
       const FastMap fm(Pj, S.degree);
       const float2 wj = tabW[jj];
       const float t = ((float)(it.j0 + jj - grp.interval * S.espan) + 0.5f) / (float)S.espan;
-      float2 m0 = make_float2(0.f, 0.f), m1 = m0;  // moments (2pa, 2pb | 2pb + 1), (2pa + 1, ...)
+      // moments (2pa, 2pb | 2pb + 1), (2pa + 1, ...), and their sums' rounding errors
+      float2 m0 = make_float2(0.f, 0.f), m1 = m0, e0 = m0, e1 = m0;
       int nr = 0;                                  // runs held in mom, the present one not counted
       int cx = kOffFrame, cy = kOffFrame;          // the present run's window centre (uniform)
       int rx = 0, ry = 0;                          // lane r: the window centre of run r
@@ -223,12 +228,46 @@ __global__ void __launch_bounds__(kMThreads, 1) k_ellip_moments(const MomentArgs
             }
           }
         };
-        // the high degrees first: the sums stay small until the last few terms, and so does their
-        // rounding (degrees 0, 2, .. in this order; the other way round every sum rounds 36 times)
+        // the high degrees first: these sums stay small, and so does their rounding
 #pragma unroll 2
-        for (int q = kEllTerms - 1; q >= kEllEven; --q) term(q, od);
+        for (int q = kEllTerms - 1; q >= kEllEven + kEllLowOdd; --q) term(q, od);
 #pragma unroll 2
-        for (int q = kEllEven - 1; q >= 0; --q) term(q, ev);
+        for (int q = kEllEven - 1; q >= kEllLowEven; --q) term(q, ev);
+        // then degrees 0 to 2, slot by slot, their sums' errors added to those of the high degrees
+        // (FastTwoSum: the lowest degree, the largest, first); ev and od end as the pixels of the pairs
+#pragma unroll
+        for (int i = 0; i < SL; ++i) {
+          float2 se[R / 2], so[R / 2];
+#pragma unroll
+          for (int r = 0; r < R / 2; ++r) se[r] = so[r] = make_float2(0.f, 0.f);
+          auto sure = [&](int q, int lq, float2 (&s)[R / 2], float2 (&acc)[R / 2][SL]) {
+            const float4 k = tab[q * NS + lane + 32 * i];
+            const float c = fmaf(fmaf(fmaf(k.w, t, k.z), t, k.y), t, k.x);
+            const float2 cc = make_float2(c, c);
+            const float2* mq = reinterpret_cast<const float2*>(mom + q * R);
+            const float2* lw = reinterpret_cast<const float2*>(low + lq * R);
+#pragma unroll
+            for (int r = 0; r < R / 2; ++r) {
+              const float2 m = mq[r], n = __ffma2_rn(cc, m, s[r]);
+              float2 e = __ffma2_rn(cc, m, sub2(s[r], n));
+              e = __ffma2_rn(cc, lw[r], e);
+              acc[r][i] = __fadd2_rn(acc[r][i], e);
+              s[r] = n;
+            }
+          };
+#pragma unroll 1
+          for (int q = 0; q < kEllLowEven; ++q) sure(q, q, se, ev);
+#pragma unroll 1
+          for (int q = 0; q < kEllLowOdd; ++q) sure(kEllEven + q, kEllLowEven + q, so, od);
+#pragma unroll
+          for (int r = 0; r < R / 2; ++r) {  // the sums, then times the sample's flux
+            const float2 p = __fadd2_rn(__fadd2_rn(se[r], so[r]), __fadd2_rn(ev[r][i], od[r][i]));
+            const float2 n = __fadd2_rn(sub2(se[r], so[r]), sub2(ev[r][i], od[r][i]));
+            const float2 wx = make_float2(wj.x, wj.x), wy = make_float2(wj.y, wj.y);
+            ev[r][i] = __ffma2_rn(p, wx, __fmul2_rn(p, wy));
+            od[r][i] = __ffma2_rn(n, wx, __fmul2_rn(n, wy));
+          }
+        }
 #pragma unroll
         for (int r = 0; r < R; ++r) {
           if (r < nr) {  // uniform
@@ -238,8 +277,7 @@ __global__ void __launch_bounds__(kMThreads, 1) k_ellip_moments(const MomentArgs
             float mx = 0.f;
 #pragma unroll
             for (int i = 0; i < SL; ++i) {
-              const float e = (r & 1) ? ev[r / 2][i].y : ev[r / 2][i].x, o = (r & 1) ? od[r / 2][i].y : od[r / 2][i].x;
-              v[i] = make_float2(e + o, e - o);
+              v[i] = (r & 1) ? make_float2(ev[r / 2][i].y, od[r / 2][i].y) : make_float2(ev[r / 2][i].x, od[r / 2][i].x);
               mx = fmaxf(mx, fmaxf(fabsf(v[i].x), fabsf(v[i].y)));
             }
             const bool small = __all_sync(0xffffffffu, mx * sc_hi < 4190000.f);
@@ -266,7 +304,8 @@ __global__ void __launch_bounds__(kMThreads, 1) k_ellip_moments(const MomentArgs
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                   if (lane + 32 * i >= NP - h) continue;
-                  const int gx = gx0 + (h ? K - 1 - pm[i] : pm[i]), gy = gy0 + (h ? K - 1 - pn[i] : pn[i]);
+                  const int e = h ? K * K - 1 - lane - 32 * i : lane + 32 * i;
+                  const int gx = gx0 + e % K, gy = gy0 + e / K;
                   const float val = h ? v[i].y : v[i].x;
                   if (gx >= 0 && gx < it.bw && gy >= 0 && gy < it.bh) {
                     int* p = boxh + gy * it.bw + gx;
@@ -286,21 +325,30 @@ __global__ void __launch_bounds__(kMThreads, 1) k_ellip_moments(const MomentArgs
         __syncwarp();
       };
       // the present run's moments into mom
-      auto close = [&]() {
+      auto close = [&](bool end) {  // end: the sample's last run, whose pixels the caller forms
         if (cx == kOffFrame) return;
-        const float m00 = __shfl_sync(0xffffffffu, m1.x, 21) + __shfl_sync(0xffffffffu, m0.y, 22);
-        if (lane == 0) m0.x = m00;
-        // ... times the sample's flux
-        mom[mrow[0] + nr] = fmaf(m0.x, wj.x, m0.x * wj.y);
-        mom[mrow[1] + nr] = m0.y * wj.x;
-        mom[mrow[2] + nr] = m1.x * wj.x;
-        mom[mrow[3] + nr] = m1.y * wj.x;
+        const float ws = __shfl_sync(0xffffffffu, m1.x, 21);  // M_00: the leading bits and the rest
+        const float wr = __shfl_sync(0xffffffffu, e1.x, 21) +
+                         (__shfl_sync(0xffffffffu, m0.y, 22) + __shfl_sync(0xffffffffu, e0.y, 22));
+        if (lane == 0) {
+          m0.x = ws;
+          e0.x = wr;
+        }
+        auto put = [&](int q, float m, float e) {
+          const float h = m + e;
+          mom[((mrow >> (8 * q)) & 0xff) * R + nr] = h;
+          low[((lrow >> (8 * q)) & 0xff) * R + nr] = (m - h) + e;
+        };
+        put(0, m0.x, e0.x);
+        put(1, m0.y, e0.y);
+        put(2, m1.x, e1.x);
+        put(3, m1.y, e1.y);
         if (lane == nr) {
           rx = cx;
           ry = cy;
         }
-        m0 = m1 = make_float2(0.f, 0.f);
-        if (++nr == R) apply();
+        m0 = m1 = e0 = e1 = make_float2(0.f, 0.f);
+        if (++nr == R && !end) apply();
       };
 
       for (int k0 = 0; k0 < it.nk; k0 += 32) {
@@ -348,7 +396,7 @@ __global__ void __launch_bounds__(kMThreads, 1) k_ellip_moments(const MomentArgs
           unsigned st = (starts >> (half * kMStage)) & ((1u << ns) - 1u);
           for (int s = 0; s < ns;) {
             if (st & 1u) {  // uniform
-              close();
+              close(false);
               cx = __shfl_sync(0xffffffffu, ci[0], half * kMStage + s);
               cy = __shfl_sync(0xffffffffu, ri[0], half * kMStage + s);
             }
@@ -357,10 +405,14 @@ __global__ void __launch_bounds__(kMThreads, 1) k_ellip_moments(const MomentArgs
             const int end = s + len;
             st >>= len - 1;
             auto add = [&](float xa, float xb, float ya, float yb) {
-              m0.x = fmaf(xa, ya, m0.x);
-              m0.y = fmaf(xa, yb, m0.y);
-              m1.x = fmaf(xb, ya, m1.x);
-              m1.y = fmaf(xb, yb, m1.y);
+              auto sum = [](float2 x, float2 y, float2& m, float2& e) {
+                const float2 n = __ffma2_rn(x, y, m);
+                e = __fadd2_rn(e, __ffma2_rn(x, y, sub2(m, n)));
+                m = n;
+              };
+              const float2 y = make_float2(ya, yb);
+              sum(make_float2(xa, xa), y, m0, e0);
+              sum(make_float2(xb, xb), y, m1, e1);
             };
             auto one = [&](int q) {
               const int o = (q >> 1) * kMPair + 2 * (q & 1);
@@ -379,7 +431,7 @@ __global__ void __launch_bounds__(kMThreads, 1) k_ellip_moments(const MomentArgs
           }
         }
       }
-      close();
+      close(true);
       if (nr > 0) apply();
     }
     __syncthreads();
