@@ -452,10 +452,10 @@ def run_gpu(args):
     peaks, peak_kind = _peaks()
     mhz = clocks["sm_mhz"] or peaks.get("sm_max_mhz", 2070.0)
     n_sm = torch.cuda.get_device_properties(dev).multi_processor_count
-    kr = statistics.median(kern.get("render_mixed", [float("nan")]))
-    # the tiles no item overlaps are zeroed by extra CTAs of the render launch (a separate
-    # launch only for a model without items); the rest merge inside the render
-    km = statistics.median(kern["merge_zero"]) if "merge_zero" in kern else 0.0
+    # the render kernel this model takes, and its tile merge (inside the render for the edge tails)
+    kname = "render_poly" if "render_poly" in kern else "render_mixed"
+    kr = statistics.median(kern.get(kname, [float("nan")]))
+    km = statistics.median(kern["merge"]) if "merge" in kern else 0.0
     d = w.model.slices[0].degree
     ns = w.model.slices[0].n_slit
     # peaks from unit counts and the sampled clock: 128 FP32 lanes per SM; FP64 from the
@@ -470,10 +470,10 @@ def run_gpu(args):
     traffic = _load_traffic()
     roof32 = {"bound": "alu", "achieved": a32 / 1e12, "peak": fp32_peak / 1e12, "unit": "TFLOP/s",
               "frac": a32 / fp32_peak, "traffic": traffic,
-              "kernel": "render_mixed", "pipe": "fp32", "kernel_ms": kr,
+              "kernel": kname, "pipe": "fp32", "kernel_ms": kr,
               "peak_basis": f"{n_sm} SMs x 128 FP32 lanes x 2 x {mhz:.0f} MHz (median SM clock under load)"}
     roof64 = {"bound": "alu", "achieved": a64 / 1e12, "peak": fp64_peak / 1e12, "unit": "TFLOP/s",
-              "frac": a64 / fp64_peak, "traffic": traffic, "kernel": "render_mixed", "pipe": "fp64", "kernel_ms": kr,
+              "frac": a64 / fp64_peak, "traffic": traffic, "kernel": kname, "pipe": "fp64", "kernel_ms": kr,
               "peak_basis": f"{n_sm} SMs x {dfma_per_clk_sm:.2f} DFMA/clk (nominal 1.25 TFLOP/s at 2070 MHz) x 2 x "
                             f"{mhz:.0f} MHz"}
     roof32["probe_tflops"] = probe["fp32"]["tflops"]
@@ -498,7 +498,7 @@ def run_gpu(args):
         "roofline": roof, "roofline_other_pipe": other,
         "fp64_renderer": {"value": fp64_value, "unit": UNIT, "ms_per_step": statistics.median(fp64_ms),
                           "speedup_mixed_over_fp64": statistics.median(fp64_ms) / ms_per_step},
-        "kernel_ms": {"render_mixed (with the tile merge and the zero tiles)": kr, "merge_zero_tiles": km},
+        "kernel_ms": {kname: kr, "merge": km},
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                 "ms_per_step": statistics.median(e2e_ms), "steps": n_e2e,
                 "note": "spectra upload + render into pinned host memory + unload per step, the next step's "

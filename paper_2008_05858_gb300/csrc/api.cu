@@ -768,35 +768,41 @@ int plan_model(Model* m) {
   // elliptical kernel has no run tiles: one item per (32-sample, 16-point) block.
   int K = 0;
   for (auto& s : m->slices) K = std::max(K, s.d.K);
-  double best = 1e300, best_tail = 1e300;
-  int bB = 1, bDX = 0, bDY = 0;
   const int variants[5][2] = {{0, 0}, {1, 1}, {1, 2}, {1, 3}, {2, 2}};
-  for (int q = 0; q <= 4 && !ellip; ++q) {  // B = 1..16
-    const int B = 1 << q;
-    int sx = 0, sy = 0;
-    for (int i = 0; i < ns; ++i) {
-      sx = std::max(sx, spans[(i * 5 + q) * 2 + 0]);
-      sy = std::max(sy, spans[(i * 5 + q) * 2 + 1]);
-    }
-    for (auto& v : variants) {
-      bool ok = true;
-      for (int k : m->Ks) ok = ok && mixed_variant_supported(k, v[0], v[1]);
-      if (!ok || sx > v[0] || sy > v[1]) continue;
-      const double ct = variant_cost(K, v[0], v[1], B);
-      if (ct < best_tail) {
-        best_tail = ct;
-        P.B_adj = B;
+  struct Variant {
+    int B = 1, DX = 0, DY = 0;
+  };
+  auto choose = [&](bool poly) {  // the cheapest variant of a kernel that holds every run
+    Variant best;
+    double least = 1e300;
+    for (int q = 0; q <= 4 && !ellip; ++q) {  // B = 1..16
+      const int B = 1 << q;
+      int sx = 0, sy = 0;
+      for (int i = 0; i < ns; ++i) {
+        sx = std::max(sx, spans[(i * 5 + q) * 2 + 0]);
+        sy = std::max(sy, spans[(i * 5 + q) * 2 + 1]);
       }
-      const double c = P.poly ? poly_variant_cost(K, v[0], v[1], B) : ct;
-      if (c < best) {
-        best = c;
-        bB = B;
-        bDX = v[0];
-        bDY = v[1];
+      for (auto& v : variants) {
+        bool ok = true;
+        for (int k : m->Ks) ok = ok && mixed_variant_supported(k, v[0], v[1]);
+        if (!ok || sx > v[0] || sy > v[1]) continue;
+        const double c = poly ? poly_variant_cost(K, v[0], v[1], B) : variant_cost(K, v[0], v[1], B);
+        if (c < least) {
+          least = c;
+          best = Variant{B, v[0], v[1]};
+        }
       }
     }
-  }
-  P.B = bB;
+    return best;
+  };
+  auto take = [&](const Variant& v) {
+    P.B = v.B;
+    P.DX = v.DX;
+    P.DY = v.DY;
+  };
+  const Variant tails = choose(false);
+  P.B_adj = tails.B;
+  take(P.poly ? choose(true) : tails);
   // The tail edges (off the centre pixel) sit at |e - f| >= 1 px from a stamp's centre, i.e. at
   // arguments w >= sqrt(log2 e) / (sqrt 2 sigma) in log2 units: when the model's widest PSF
   // keeps that at or above the cheaper rational's lower end (sigma <= 2.12 px), the separable
@@ -808,8 +814,6 @@ int plan_model(Model* m) {
     const double limit = kSqrtLog2eD / (std::sqrt(2.0) * (double)kTailFarMinArg);
     P.far_tails = !ellip && smax <= limit * (1.0 - 1e-3) ? 1 : 0;
   }
-  P.DX = bDX;
-  P.DY = bDY;
   P.max_deg = 0;
   for (auto& s : m->slices) P.max_deg = std::max(P.max_deg, s.d.degree);
 
@@ -819,7 +823,7 @@ int plan_model(Model* m) {
 
   // ---- items: (32-sample blocks) x (16-point blocks); at most 16 warp tasks (<= 512 runs,
   // which keeps the fixed-point low words of a box below 2^31) and a box that fits on chip
-  for (int jb_cap = 8; jb_cap >= 1; P.emom ? P.emom = 0 : jb_cap /= 2) {
+  auto lay_out = [&](int jb_cap) {  // the items at up to jb_cap sample blocks each; whether they fit
     int64_t store = 0;
     P.items.clear();
     P.groups.clear();
@@ -899,14 +903,31 @@ int plan_model(Model* m) {
              : P.poly ? poly_smem_bytes(area, P.JB, P.nk_max, P.max_deg + 1)
                      : mixed_smem_bytes(area, P.JB, P.nk_max, P.B, P.max_deg + 1);
     P.smem_mom = P.emom ? ellip_moment_smem(K_mom, area_mom, P.nk_mom, P.max_deg + 1) : 0;
-    // the polynomial kernel's warps take eight samples each through the whole slit: a grid that
-    // would not fill the GPU gets items of one 32-sample block (a sample octet per warp)
-    const bool thin = P.poly && jb_cap > 1 && P.JB > 1 && (int)P.items.size() < kPolyWave;
-    if ((int)std::max(P.smem, P.smem_mom) + kStaticSmemReserve <= optin && !thin) break;
-    if (jb_cap == 1 && !P.emom)
+    return (int)std::max(P.smem, P.smem_mom) + kStaticSmemReserve <= optin;
+  };
+  // Boxes too large for a kernel's shared memory get fewer sample blocks; where one block is still too
+  // much, the kernel that needs less beside the box: stamp by stamp instead of on moments, the edge
+  // tails (13 KB beside one block's box) instead of the polynomials (34 KB).
+  int jb = 8;
+  auto shrink = [&]() {
+    for (jb = 8; !lay_out(jb); jb /= 2)
+      if (jb == 1) return false;
+    return true;
+  };
+  while (!shrink()) {
+    if (P.emom) {
+      P.emom = 0;
+    } else if (P.poly) {
+      P.poly = 0;
+      take(tails);
+    } else {
       return fail(E2E_EINVAL, "trace footprint of a work item exceeds on-chip memory (area " +
                                   std::to_string(P.max_area) + " px)");
+    }
   }
+  // the polynomial kernel's warps take eight samples each through the whole slit: a grid that would
+  // not fill the GPU gets items of one 32-sample block (a sample octet per warp)
+  while (P.poly && jb > 1 && P.JB > 1 && (int)P.items.size() < kPolyWave) lay_out(jb /= 2);
   P.NB = 1;
   if (int rc1 = plan_bands_and_tiles(m); rc1 != E2E_OK) return rc1;
   if (P.emom) {
@@ -1156,7 +1177,7 @@ int render_impl(e2e_ctx* ctx, Model* m, int n_spec, const uint64_t* spec_ids, in
     }
   } else {
     for (auto& g : P.groups) {
-      KernelTimer kt(ctx, st, tab ? "render_table" : g.mom ? "render_moments" : ellip ? "render_ellip" : "render_mixed");
+      KernelTimer kt(ctx, st, tab ? "render_table" : g.mom ? "render_moments" : ellip ? "render_ellip" : "render_poly");
       E2E_CK(launch_items(ctx, m, g.K, g.first, g.count, d_table, store, st));
     }
     KernelTimer kt(ctx, st, "merge");
@@ -1854,6 +1875,7 @@ int static_scratch_address(int device, void** out) {
   return E2E_OK;
 }
 
+
 size_t align256(size_t n) { return (n + 255) & ~(size_t)255; }
 }  // namespace
 
@@ -1913,7 +1935,7 @@ int e2e_render_static(e2e_ctx* ctx, uint64_t model_id, int32_t n_spec, const uin
   if (ctx->opts.kernel_timing) reset_timing(ctx);
   if (ctx->d_err) E2E_CK(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), st));
   for (auto& grp : P.groups) {
-    KernelTimer kt(ctx, st, "render_mixed");
+    KernelTimer kt(ctx, st, P.poly ? "render_poly" : "render_mixed");
     E2E_CK(launch_items(ctx, m, grp.K, grp.first, grp.count, d_table, store, st));
   }
   {
