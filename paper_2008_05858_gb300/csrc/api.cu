@@ -607,9 +607,7 @@ int plan_bands_and_tiles(Model* m) {
   if (rc == E2E_OK) rc = upload(&P.d_tile_of, tile_of.data(), tile_of.size());
   if (rc == E2E_OK) rc = upload(&P.d_grid_off, grid_off.data(), grid_off.size());
   if (rc == E2E_OK) rc = upload(&P.d_zero_tiles, zero_tiles.data(), zero_tiles.size());
-  if (rc != E2E_OK) return rc;
-  P.ok = true;
-  return E2E_OK;
+  return rc;
 }
 
 // Wavelength samples between two nodes of an elliptical slice's table (a multiple of 32), or 0
@@ -729,7 +727,11 @@ int plan_model(Model* m) {
   Plan& P = m->plan;
   const int ns = (int)m->slices.size();
   const bool ellip = m->psf != E2E_PSF_SEPARABLE;  // item shape of the non-separable kernels
-  if (ns == 0) return plan_bands_and_tiles(m);
+  if (ns == 0) {
+    const int rc = plan_bands_and_tiles(m);
+    P.ok = rc == E2E_OK;
+    return rc;
+  }
   if (int rc0 = build_sample_tables(m); rc0 != E2E_OK) return rc0;
   if (int rc0 = build_ellip_nodes(m); rc0 != E2E_OK) return rc0;
   // ---- device pass: exact window origins of every stamp
@@ -945,8 +947,9 @@ int plan_model(Model* m) {
         P.egroups.back().count++;
       }
     }
-    return upload(&P.d_egroups, P.egroups.data(), P.egroups.size());
+    if (int rc1 = upload(&P.d_egroups, P.egroups.data(), P.egroups.size()); rc1 != E2E_OK) return rc1;
   }
+  P.ok = true;  // last: a plan that lacks any of its arrays is never used
   return E2E_OK;
 }
 
@@ -1964,6 +1967,7 @@ int e2e_render_adjoint(e2e_ctx* ctx, uint64_t model_id, int32_t n_spec, const ui
   if (m->psf != E2E_PSF_SEPARABLE) return fail(E2E_EINVAL, "the adjoint supports the separable PSF");
   if (reinterpret_cast<uintptr_t>(frozen_windows) % 8 != 0) return fail(E2E_EINVAL, "frozen_windows must be 8-byte aligned");
   const Plan& P = m->plan;
+  if (!P.ok) return fail(E2E_EINVAL, "model has no mixed-precision plan");
   std::vector<int64_t> pitch(m->n_det);
   for (int d = 0; d < m->n_det; ++d) {
     if (!dldi[d]) return fail(E2E_EINVAL, "null dL/dI frame");
