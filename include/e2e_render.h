@@ -177,10 +177,10 @@ const char* e2e_last_error(void);
  * of every slice (degree + 3) x 16 bytes of precomputed mapping coefficients and PSF constants
  * (261 MB for a 9216^2 frame of 340 slices x 6000 samples at degree 5); a separable model whose
  * widths stay >= 1 px and windows K >= 3 adds its pixel-integral polynomials, 448 bytes per sample
- * at K = 11 (0.91 GB for that frame; left out where the device has no room for them); an
- * elliptical model's slices whose widths stay >= 1.3 px and vary slowly from sample to sample add
- * the pixel integrals' coefficients at nodes along them (25 KB per node at K = 13, a node per
- * hundred samples or so); the tabulated PSF adds its coefficient tables.
+ * at K = 11 (0.91 GB for that frame; left out where they would take more than a quarter of the
+ * device's free memory); an elliptical model's slices whose widths stay >= 1.3 px and vary slowly
+ * from sample to sample add the pixel integrals' coefficients at nodes along them (25 KB per node
+ * at K = 13, a node per hundred samples or so); the tabulated PSF adds its coefficient tables.
  * Errors: E2E_EINVAL, E2E_ENOMEM, E2E_ECUDA. */
 int e2e_load_model(e2e_ctx* ctx, const e2e_model_desc* desc, uint64_t* model_id);
 int e2e_unload_model(e2e_ctx* ctx, uint64_t model_id);

@@ -685,8 +685,9 @@ int build_sample_tables(Model* m) {
     total += (int64_t)m->dev[i].n_lambda * (m->dev[i].degree + 3);
     max_lambda = std::max(max_lambda, m->dev[i].n_lambda);
   }
-  // polynomial pixel integrals, where the model's narrowest PSF allows them, in the same
-  // allocation; a device without room for them renders from the edge tails instead
+  // polynomial pixel integrals, where the model's narrowest PSF allows them, in the same allocation;
+  // where they would take more than a quarter of the device's free memory the model renders from the
+  // edge tails instead.  The tables it has are given up only once the larger ones exist.
   std::vector<int64_t> poff(ns);
   int64_t ptotal = 0;
   bool can = m->psf == E2E_PSF_SEPARABLE, poly = true;
@@ -698,18 +699,24 @@ int build_sample_tables(Model* m) {
     ptotal += (int64_t)s.n_lambda * poly_row_f4(s.K);
   }
   poly = poly && can;
-  if (poly && !m->has_poly) {  // an update widened the PSF: make room for the polynomials
-    cudaFree(m->d_stab);
-    m->d_stab = nullptr;
-  }
-  if (!m->d_stab) {
-    if (poly && cudaMalloc((void**)&m->d_stab, (size_t)(total + ptotal) * sizeof(float4)) == cudaSuccess) {
+  if (poly && !m->has_poly) {  // at load, or when an update has widened the PSF
+    const size_t bytes = (size_t)(total + ptotal) * sizeof(float4);
+    float4* both = nullptr;
+    size_t room = 0, all = 0;
+    E2E_CK(cudaMemGetInfo(&room, &all));
+    if (bytes <= room / 4) {  // the rest is for frames, spectra, a render's boxes and other models
+      if (cudaMalloc((void**)&both, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        both = nullptr;
+      }
+    }
+    if (both) {
+      cudaFree(m->d_stab);
+      m->d_stab = both;
       m->has_poly = true;
-    } else {
-      cudaGetLastError();
-      E2E_CK(cudaMalloc((void**)&m->d_stab, (size_t)total * sizeof(float4)));
     }
   }
+  if (!m->d_stab) E2E_CK(cudaMalloc((void**)&m->d_stab, (size_t)total * sizeof(float4)));
   poly = poly && m->has_poly;
   for (int i = 0; i < ns; ++i) m->dev[i].samples = m->d_stab + off[i];
   m->plan.poly = poly ? 1 : 0;

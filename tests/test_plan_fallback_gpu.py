@@ -1,5 +1,6 @@
 """Separable models that the polynomial kernel must not cost what the edge tails had: a work item whose
-box leaves no room for its exchange renders from the tails, at load and after an update, and back."""
+box leaves no room for its exchange renders from the tails, at load and after an update, and back; so
+does a model whose tables a nearly full device would not spare."""
 import numpy as np
 import pytest
 
@@ -50,3 +51,33 @@ def test_box_too_large_for_the_polynomials(renderer):
         _check(renderer, mid, sids, w, "render_mixed")
     finally:
         renderer.unload_model(mid)
+
+
+def test_no_polynomials_on_a_full_device(renderer):
+    # 320,000 samples: 41 MB of sample tables, 143 MB of polynomials, which a device with 0.4 GB left
+    # does not spare (more than a quarter); an update there keeps the tables the model has
+    w = W.small_config(seed=62, orders=2, fibers=2, slices=2, n_lambda=40000, n_slit=2, width=400, height=160)
+    narrow = W.Workload(w.name, w.model.copy(), w.spectra, w.out_dtype, w.precision)
+    for s in narrow.model.slices:
+        s.sigma_x, s.sigma_y = 0.5 * s.sigma_x, 0.5 * s.sigma_y
+    first = renderer.load_model(narrow.model)  # below 1 px: no polynomials
+    sids = renderer.load_spectra(w)
+    renderer.render(first, sids, "mixed", "f32")
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    hold = torch.empty(free - (400 << 20), dtype=torch.uint8, device="cuda:0")
+    second = 0
+    try:
+        second = renderer.load_model(w.model)
+        _check(renderer, second, sids, w, "render_mixed")
+        cx, cy, sx, sy = renderer.params(first)
+        renderer.update(first, cx, cy, 2.0 * sx, 2.0 * sy)
+        _check(renderer, first, sids, w, "render_mixed")
+        del hold
+        torch.cuda.empty_cache()
+        renderer.update(first, cx, cy, 2.0 * sx, 2.0 * sy)
+        _check(renderer, first, sids, w, "render_poly")
+    finally:
+        for mid in (first, second):
+            if mid:
+                renderer.unload_model(mid)
