@@ -106,7 +106,11 @@ struct Plan {
   int n_zero_tiles = 0;
 };
 
-constexpr int kPolyWave = 152 * 4;  // CTAs of the polynomial kernel the GPU holds at once
+// Items below which the polynomial render's items are cut to one sample block each: four for each of
+// 152 SMs, whatever number of CTAs an SM holds.  At 504 items of two blocks (4096 x 1024 frame, 8 traces
+// of 4000 x 16 stamps) cutting takes K = 13 from 88 to 82 us and K = 9 from 66 to 61 (three CTAs an SM),
+// and costs K = 11 (four) 60 -> 66.
+constexpr int kPolyWave = 152 * 4;
 constexpr int kBands = 16;  // y-bands of a frame rendered into host memory
 
 struct Model {
