@@ -6,9 +6,11 @@
 //   b = 0:      differences over the pixel's left and right edge of A(x) = int f(x, y) dy over its
 //               rows and A's derivatives (A' = -x A / vx + P12/P22 [f] over the rows' ends),
 //   a = 0:      the same along y;  a = b = 0: 12-point Gauss-Legendre over A.
-// They are then expanded in T_p(2 fx) T_q(2 fy) and cut after p + q = kEllDegree.  About 6e5
-// operations per node of a 13 x 13 window; a node per ~100 samples costs the load of an order-slice
-// of 8000 samples ~0.1 ms.
+// They are then expanded in T_p(2 fx) T_q(2 fy) and cut after p + q = kEllDegree.  FP64 arithmetic
+// bounds it (1/64 of the FP32 rate): some 7000 operations a pixel pair, half of them the corners'
+// recurrences.  24 slices of 8000 samples, K = 13, a node per 64 samples: 6.5 ms, 0.27 ms a slice,
+// of a load of 11 ms (11.2 and 16 ms with the recurrences' divisions as divisions).  An update of the
+// coefficients pays it again.
 #include "e2e_kernels.h"
 #include "ellip_moments.cuh"
 #include "mixed_common.cuh"
@@ -35,6 +37,10 @@ __device__ constexpr double kChebOf[kEllTaylor + 1][kEllDegree + 1] = {
     {5.507469177246094e-05, 0, 9.441375732421875e-05, 0, 5.900859832763672e-05, 0, 2.6226043701171875e-05, 0, 7.867813110351562e-06, 0, 1.430511474609375e-06},
     {0, 5.1140785217285156e-05, 0, 3.835558891296387e-05, 0, 2.130866050720215e-05, 0, 8.52346420288086e-06, 0, 2.3245811462402344e-06, 0},
     {1.2785196304321289e-05, 0, 2.2374093532562256e-05, 0, 1.4916062355041504e-05, 0, 7.458031177520752e-06, 0, 2.7120113372802734e-06, 0, 6.780028343200684e-07}};
+
+// 1 / n: an FP64 division is some ten FP64 instructions, and the recurrences divide by their index.
+__device__ constexpr double kRecip[kEllTaylor + 2] = {0.0, 1.0, 1.0 / 2, 1.0 / 3, 1.0 / 4, 1.0 / 5, 1.0 / 6, 1.0 / 7, 1.0 / 8,
+                                                      1.0 / 9, 1.0 / 10, 1.0 / 11, 1.0 / 12, 1.0 / 13, 1.0 / 14, 1.0 / 15};
 
 // P(a < Z < b) of a standard normal, tails subtracted on one side of the mean.
 __device__ __forceinline__ double between(double a, double b) {
@@ -75,7 +81,7 @@ __global__ void __launch_bounds__(128) k_ellip_nodes(const DevSlice* __restrict_
   for (int a = 0; a <= N; ++a)
 #pragma unroll 1
     for (int b = 0; b <= N - a; ++b) c[a][b] = 0.0;
-  const double inv_det = rs2pi * rs2pi / sqrt(det);
+  const double inv_det = rs2pi * rs2pi / sqrt(det), ivx = 1.0 / vx, ivy = 1.0 / vy, qx = P12 / P22, qy = P12 / P11;
   // A's and B's derivative sources: differences over the pixel's rows (columns) of h_(a,0) (h_(0,b))
   double fa[2][N + 1], fb[2][N + 1];
 #pragma unroll 1
@@ -89,7 +95,7 @@ __global__ void __launch_bounds__(128) k_ellip_nodes(const DevSlice* __restrict_
     h[0] = inv_det * exp(-0.5 * (x * L1 + y * L2));
     h[1] = -L2 * h[0];
 #pragma unroll 1
-    for (int b = 1; b < N; ++b) h[b + 1] = -(L2 * h[b] + P22 * h[b - 1]) / (double)(b + 1);
+    for (int b = 1; b < N; ++b) h[b + 1] = -(L2 * h[b] + P22 * h[b - 1]) * kRecip[b + 1];
 #pragma unroll 1
     for (int b = 0; b <= N; ++b) {
       hp[b] = 0.0;
@@ -98,12 +104,12 @@ __global__ void __launch_bounds__(128) k_ellip_nodes(const DevSlice* __restrict_
 #pragma unroll 1
     for (int a = 0; a < N; ++a) {
       fa[ix][a] += iy ? h[0] : -h[0];
-      const double ra = 1.0 / (double)(a + 1);
+      const double ra = kRecip[a + 1];
       double left = 0.0;  // row a, column b - 1
 #pragma unroll 1
       for (int b = 0; b <= N - a - 1; ++b) {
         const double v = h[b];
-        if (b + 1 <= N - a - 1) c[a + 1][b + 1] += sg * v * ra / (double)(b + 1);
+        if (b + 1 <= N - a - 1) c[a + 1][b + 1] += sg * v * ra * kRecip[b + 1];
         const double nx = -(L1 * v + P11 * hp[b] + P12 * left) * ra;
         hp[b] = v;
         left = v;
@@ -120,10 +126,11 @@ __global__ void __launch_bounds__(128) k_ellip_nodes(const DevSlice* __restrict_
     double alp = 0.0, bep = 0.0;
 #pragma unroll 1
     for (int a = 1; a <= N; ++a) {
-      c[a][0] += sg * al / (double)a;
-      c[0][a] += sg * be / (double)a;
-      const double an = (-(x * al + alp) / vx + P12 / P22 * fa[s][a - 1]) / (double)a;
-      const double bn = (-(y * be + bep) / vy + P12 / P11 * fb[s][a - 1]) / (double)a;
+      const double ia = kRecip[a];
+      c[a][0] += sg * al * ia;
+      c[0][a] += sg * be * ia;
+      const double an = (-(x * al + alp) * ivx + qx * fa[s][a - 1]) * ia;
+      const double bn = (-(y * be + bep) * ivy + qy * fb[s][a - 1]) * ia;
       alp = al;
       al = an;
       bep = be;
@@ -134,7 +141,7 @@ __global__ void __launch_bounds__(128) k_ellip_nodes(const DevSlice* __restrict_
 #pragma unroll 1
   for (int q = 0; q < kGl12; ++q) {
     const double u = X + kGl12T[q];
-    g += kGl12W[q] * exp(-0.5 * u * u / vx) * between((Y - 0.5 - bx * u) * isx, (Y + 0.5 - bx * u) * isx);
+    g += kGl12W[q] * exp(-0.5 * u * u * ivx) * between((Y - 0.5 - bx * u) * isx, (Y + 0.5 - bx * u) * isx);
   }
   c[0][0] = g * rs2pi / sqrt(vx);
   // d/dfx = -d/dX: odd a + b change sign; rows then columns into T_p(2 fx) T_q(2 fy)
