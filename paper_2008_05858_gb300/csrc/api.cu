@@ -472,7 +472,7 @@ int build_psf_tables(Model* m) {
   if (rc == E2E_OK && (cudaMalloc((void**)&m->d_T64, std::max<int64_t>(1, tab) * sizeof(double)) != cudaSuccess ||
                        cudaMalloc((void**)&m->d_T32, std::max<int64_t>(1, tab32) * sizeof(float)) != cudaSuccess))
     rc = fail(E2E_ENOMEM, "PSF tables");
-  if (rc == E2E_OK) {  // the FP32 rows' padding is never read; zero it all the same
+  if (rc == E2E_OK) {  // whole warps read the FP32 rows, padding included: it has to be zero
     const cudaError_t e = cudaMemset(m->d_T32, 0, std::max<int64_t>(1, tab32) * sizeof(float));
     if (e != cudaSuccess) rc = cuda_fail(e, "PSF tables");
   }

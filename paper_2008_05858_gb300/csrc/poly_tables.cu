@@ -6,7 +6,7 @@
 // multiplications per half pixel), because its error would scale every coefficient; the Hermite
 // recurrences and their differences (pixels near the centre), the Gauss-Legendre sums (wing
 // pixels) and the Chebyshev truncation run in FP32, where they add a few 1e-8: the table of a
-// 2.04e6-sample model costs a fraction of a millisecond instead of ~10 ms all in FP64.
+// 2.04e6-sample model (K = 11) costs 1.4 ms instead of ~10 ms all in FP64.
 #include "e2e_kernels.h"
 #include "poly_tables.cuh"
 #include "quad_coeffs.h"

@@ -1,6 +1,6 @@
 // The separable-PSF mixed-precision render kernel on edge tails (see render_mixed.cu), for models
-// with widths below 1 px or K = 1 (wider PSFs take render_poly.cuh: 4096^2 frame of 40 x 4000 x 32
-// stamps, K = 11, 0.32 ms here, 0.24 ms there), as a template
+// with widths below 1 px or K = 1, and boxes that leave the other kernel no room (wider PSFs take
+// render_poly.cuh, with both kernels' times), as a template
 // instantiated by render_mixed.cu (production) and render_mixed_check.cu (debug checks).
 #pragma once
 #include "e2e_device.cuh"

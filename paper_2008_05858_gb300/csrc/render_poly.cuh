@@ -9,21 +9,21 @@
 // walks all the item's slit points with them, so that a lane loads its coefficients once per
 // sample and holds them in registers: lane (axis, half) of the quad evaluates half the pixel pairs
 // of one axis of every stamp, at K = 11 some two dozen packed and scalar operations and, for the
-// slopes of its two wing pairs, four exponentials (3 % of the 9216^2 frame below, 3.79 -> 3.91 ms
-// with its merge; without them narrow PSFs' wings miss the bound, poly_tables.cuh).  The quad's
+// slopes of its two wing pairs, four exponentials (1.5 % of the 9216^2 frame, 3.71 -> 3.77 ms with
+// its merge; without them narrow PSFs' wings miss the bound, poly_tables.cuh).  The quad's
 // profiles go through shared memory, and each lane adds one quadrant of the tile's outer product.
 // The tiles are merged by a kernel of their own: the last CTA of a tile merging it while three
 // others hold the SM cost more (0.5 ms of a 9216^2 frame) than the separate launch (0.3 ms).
 //
-// Measured on the 9216^2 frame of 340 slices x 6000 x 64 stamps: 3.4 ms (the edge tails 5.1 ms),
-// 4096^2 frame of 40 x 4000 x 32 0.21 ms (0.31).  Per stamp ~20 warp-instructions; the shared-
-// memory pipe is busy 78 % of the time, the FMA pipe 44 %, issue slots 60 %; four CTAs of 128
-// threads per SM (128 registers) leave the rest to latency.  Five CTAs spill (5.8 ms).  Windows of 9,
-// 13 and 15 px spill at four already (32 to 96 bytes a thread; the wide ones hold four pixel pairs'
-// coefficients and a tile quadrant of 7 x 7 pixels) and run three to an SM, with up to 168
-// registers: on the 4096^2 frame
-// K = 13 451 -> 377 us, K = 15 1237 -> 1178, K = 9 199 -> 190; 2473^2 frame of 40 x 3989 x 59 stamps,
-// K = 13, 768 -> 560 us (the edge tails 686).
+// Measured on the benchmark's 9216^2 frame of 340 slices x 6000 x 64 stamps: 3.76 ms (the edge tails
+// with their merge 5.2 ms), 4096^2 frame of 40 x 4000 x 32 with its merge 0.24 ms (0.33).  Per stamp
+// 21 warp-instructions; the shared-memory pipe is busy 73 % of the time, the FMA pipe 46 %, issue
+// slots 61 %; four CTAs of 128 threads per SM (128 registers) leave the rest to latency.  Five CTAs
+// spill.  Windows of 9, 13 and 15 px spill at four already (the wide ones hold four pixel pairs'
+// coefficients and a tile quadrant of 7 x 7 pixels) and run three to an SM, with up to 168 registers.
+// It is the faster one at every size: 4096^2 frame of 40 traces x 4000 samples, K = 15, 8 / 32 / 64
+// slit points 380 / 1250 / 2440 us against 499 / 1631 / 3175 for the edge tails, K = 11, 1 / 4 / 7
+// points 143 / 170 / 201 against 155 / 180 / 252.
 #pragma once
 #include <type_traits>
 
@@ -305,18 +305,16 @@ __global__ void __launch_bounds__(kPThreads, poly_ctas(K)) k_render_poly(const M
               float* row = wrow + (parity + e) * kPBuf;
 #pragma unroll
               for (int s = 0; s < NS; ++s) {
-                float2 v;  // G(i + f), G(i - f)
+                const float Ew = p[e][s].x * mult[e];
+                float v0 = fmaf(fw[e], p[e][s].y, Ew), v1 = fmaf(-fw[e], p[e][s].y, Ew);  // G(i + f), G(i - f)
                 if (poly_wing(K, s)) {
-                  const float f = axis ? st[e].y : st[e].x, t = f * wing[s];
-                  v = __ffma2_rn(make_float2(p[e][s].y, p[e][s].y), make_float2(f, -f), make_float2(p[e][s].x, p[e][s].x));
-                  v = __fmul2_rn(v, __fmul2_rn(make_float2(mult[e], mult[e]), make_float2(ex2_approx(-t), ex2_approx(t))));
-                } else {
-                  const float Ew = p[e][s].x * mult[e];
-                  v = make_float2(fmaf(fw[e], p[e][s].y, Ew), fmaf(-fw[e], p[e][s].y, Ew));
+                  const float t = (axis ? st[e].y : st[e].x) * wing[s];
+                  v0 *= ex2_approx(-t);
+                  v1 *= ex2_approx(t);
                 }
                 if (2 * s + 1 <= H || half == 0) {  // half 1 has one pair fewer when H is even
-                  row[2 * s] = v.x;
-                  row[K - 1 - 2 * half - 2 * s] = v.y;
+                  row[2 * s] = v0;
+                  row[K - 1 - 2 * half - 2 * s] = v1;
                 }
               }
             }
