@@ -733,6 +733,25 @@ int build_sample_tables(Model* m) {
   return E2E_OK;
 }
 
+size_t align256(size_t n) { return (n + 255) & ~(size_t)255; }
+
+// What e2e_render_static lays out in its buffer: flux table | pitches | destination pointers | box
+// store [| blazed spectra | original flux table].
+struct StaticLayout {
+  size_t table, pitch, dst, store, blaze, tin, need;
+};
+StaticLayout static_layout(const Model& m, int64_t store_elems) {
+  StaticLayout L{};
+  const size_t n = m.slices.size() * sizeof(double*);
+  L.pitch = align256(L.table + n);
+  L.dst = align256(L.pitch + (size_t)m.n_det * sizeof(int64_t));
+  L.store = align256(L.dst + (size_t)m.n_det * sizeof(void*));
+  L.blaze = align256(L.store + (size_t)store_elems * sizeof(float2));
+  L.tin = align256(L.blaze + (m.has_blaze ? (size_t)m.n_bins * sizeof(double) : 0));
+  L.need = m.has_blaze ? L.tin + n : L.blaze;
+  return L;
+}
+
 int plan_model(Model* m) {
   NvtxRange nvtx_("e2e plan");
   Plan& P = m->plan;
@@ -939,8 +958,30 @@ int plan_model(Model* m) {
     }
   }
   // the polynomial kernel's warps take eight samples each through the whole slit: a grid that would
-  // not fill the GPU gets items of one 32-sample block (a sample octet per warp)
-  while (P.poly && jb > 1 && P.JB > 1 && (int)P.items.size() < kPolyWave) lay_out(jb /= 2);
+  // not fill the GPU gets items of one 32-sample block (a sample octet per warp), as long as the boxes,
+  // which overlap more then, stay within the fixed-scratch render's buffer
+  auto fits_static = [&]() { return static_layout(*m, P.store_elems).need <= E2E_STATIC_SCRATCH_BYTES; };
+  while (P.poly && jb > 1 && P.JB > 1 && (int)P.items.size() < kPolyWave) {
+    const bool fit = fits_static();
+    lay_out(jb / 2);
+    if (fit && !fits_static()) {
+      lay_out(jb);
+      break;
+    }
+    jb /= 2;
+  }
+  // ... and where they do not, but the tails' larger items would, the model takes those
+  if (P.poly && !fits_static() && (jb < 8 || tails.B != P.B)) {
+    const Variant mine{P.B, P.DX, P.DY};
+    const int jb_mine = jb;
+    P.poly = 0;
+    take(tails);
+    if (!shrink() || !fits_static()) {
+      P.poly = 1;
+      take(mine);
+      lay_out(jb = jb_mine);
+    }
+  }
   P.NB = 1;
   if (int rc1 = plan_bands_and_tiles(m); rc1 != E2E_OK) return rc1;
   if (P.emom) {
@@ -1888,9 +1929,6 @@ int static_scratch_address(int device, void** out) {
   *out = p;
   return E2E_OK;
 }
-
-
-size_t align256(size_t n) { return (n + 255) & ~(size_t)255; }
 }  // namespace
 
 int e2e_render_static(e2e_ctx* ctx, uint64_t model_id, int32_t n_spec, const uint64_t* spec_ids, int32_t dtype,
@@ -1914,29 +1952,21 @@ int e2e_render_static(e2e_ctx* ctx, uint64_t model_id, int32_t n_spec, const uin
   std::vector<const double*> table;
   int rc = resolve_flux(ctx, m, n_spec, spec_ids, table);
   if (rc != E2E_OK) return rc;
-  // layout in the fixed buffer: flux table | pitches | destination pointers | box store
-  // [| blazed spectra | original flux table]
-  const size_t off_table = 0;
-  const size_t off_pitch = align256(off_table + table.size() * sizeof(double*));
-  const size_t off_dst = align256(off_pitch + pitch.size() * sizeof(int64_t));
-  const size_t off_store = align256(off_dst + (size_t)m->n_det * sizeof(void*));
-  const size_t off_blaze = align256(off_store + (size_t)P.store_elems * sizeof(float2));
-  const size_t off_tin = align256(off_blaze + (m->has_blaze ? (size_t)m->n_bins * sizeof(double) : 0));
-  const size_t need = m->has_blaze ? off_tin + table.size() * sizeof(double*) : off_blaze;
-  if (need > E2E_STATIC_SCRATCH_BYTES)
-    return fail(E2E_ETOOBIG, "model needs " + std::to_string(need) + " bytes of scratch; the fixed buffer holds " +
+  const StaticLayout L = static_layout(*m, P.store_elems);
+  if (L.need > E2E_STATIC_SCRATCH_BYTES)
+    return fail(E2E_ETOOBIG, "model needs " + std::to_string(L.need) + " bytes of scratch; the fixed buffer holds " +
                                  std::to_string((size_t)E2E_STATIC_SCRATCH_BYTES));
   void* base = nullptr;
   rc = static_scratch_address(ctx->device, &base);
   if (rc != E2E_OK) return rc;
   unsigned char* b = static_cast<unsigned char*>(base);
-  const double** d_table = reinterpret_cast<const double**>(b + off_table);
-  int64_t* d_pitch = reinterpret_cast<int64_t*>(b + off_pitch);
-  void** d_dst = reinterpret_cast<void**>(b + off_dst);
-  float2* store = reinterpret_cast<float2*>(b + off_store);
+  const double** d_table = reinterpret_cast<const double**>(b + L.table);
+  int64_t* d_pitch = reinterpret_cast<int64_t*>(b + L.pitch);
+  void** d_dst = reinterpret_cast<void**>(b + L.dst);
+  float2* store = reinterpret_cast<float2*>(b + L.store);
   cudaStream_t st = (cudaStream_t)stream;
   if (m->has_blaze && !table.empty()) {
-    rc = blaze_into(m, table, reinterpret_cast<double*>(b + off_blaze), reinterpret_cast<const double**>(b + off_tin),
+    rc = blaze_into(m, table, reinterpret_cast<double*>(b + L.blaze), reinterpret_cast<const double**>(b + L.tin),
                     st);
     if (rc != E2E_OK) return rc;
   }
