@@ -59,13 +59,16 @@ def _peaks():
 
 
 # FP32 FLOP of one separable stamp of window K and degree d, counted algorithmically (an FMA
-# is 2 FLOP, an SFU operation 1): 2(K+1) pixel-edge tail evaluations at 28 FLOP each (the
-# double-float edge argument: 6; its exact square: 3; the exponential: 1 + 2; the (4,5)
-# rational: 18 - 2 = 16, with its reciprocal), 2K edge differences, the K^2 products with the
-# weight folded in, accumulated by FMA (2 K^2), and the mapping's Horner in s of both
-# coordinates (2d FMAs; evaluated in double-float FP32 arithmetic, counted once).
-def fp32_flop_per_stamp(K: int, d: int = 5) -> float:
-    return 2 * (K + 1) * 28 + 2 * K + 2 * K * K + 4 * d
+# is 2 FLOP, an SFU operation 1): its 2K pixel integrals, the K^2 products with the weight folded
+# in, accumulated by FMA (2 K^2), and the mapping's Horner in s of both coordinates (2d FMAs,
+# counted once).  The pixel integrals of the polynomial render: per axis f^2 and K // 2 + 1 pixel
+# pairs of two Horner sums of five terms (16), f O (1, shared: the weight times f), E +- f O with the
+# weight (5); a wing pair's slopes (2 exponentials and 4 products) are left out.  Of the edge tails:
+# 2(K+1) edges at 28 FLOP (the double-float edge argument: 6; its exact square: 3; the exponential:
+# 1 + 2; the (4,5) rational: 18 - 2 = 16, with its reciprocal) and 2K edge differences.
+def fp32_flop_per_stamp(K: int, d: int = 5, poly: bool = False) -> float:
+    pixels = 2 * (1 + 1 + (K // 2 + 1) * 21) if poly else 2 * (K + 1) * 28 + 2 * K
+    return pixels + 2 * K * K + 4 * d
 
 
 # FP64 FMAs of one stamp: the per-sample Horner in lambda of the coefficients of s (2 n_c per
@@ -465,7 +468,7 @@ def run_gpu(args):
     fp32_peak = n_sm * 128 * 2 * mhz * 1e6
     fp64_peak = n_sm * dfma_per_clk_sm * 2 * mhz * 1e6
     probe = pipe_rates(B, dev)
-    a32 = fp32_flop_per_stamp(K, d) * stamps_rank / (kr * 1e-3)
+    a32 = fp32_flop_per_stamp(K, d, kname == "render_poly") * stamps_rank / (kr * 1e-3)
     a64 = fp64_fma_per_stamp(d, ns) * 2 * stamps_rank / (kr * 1e-3)
     traffic = _load_traffic()
     roof32 = {"bound": "alu", "achieved": a32 / 1e12, "peak": fp32_peak / 1e12, "unit": "TFLOP/s",
