@@ -23,9 +23,9 @@
 //   T(f) = G(i + f) 2^(f k_i),   k_i = log2(e) i / sigma^2  (poly_wing_rate),
 //
 // which varies by a few tens of a percent and needs a term less, and the kernel multiplies
-// T(f) = E + f O and T(-f) = E - f O (with the weight) by 2^(-f k_i) and 2^(f k_i).  Worst of 3072 single stamps, K = 11,
-// in parts of the bound: 1.64, 1.37, 1.02, 1.03 at sigma = 1.0, 1.1, 1.2, 1.3 before,
-// 0.64, 0.54, 0.52, 0.44 now (the edge tails 0.64, 0.72, 0.85, 0.84).
+// T(f) = E + f O and T(-f) = E - f O (with the weight) by 2^(-f k_i) and 2^(f k_i).  Worst of 3072
+// single stamps, K = 11, in parts of the bound: 1.64, 1.37, 1.02, 1.03 at sigma = 1.0, 1.1, 1.2, 1.3
+// as a plain E - f O, 0.64, 0.54, 0.52, 0.44 so (the edge tails 0.64, 0.72, 0.85, 0.84).
 #pragma once
 #include "e2e_device.cuh"
 

@@ -2,7 +2,7 @@
 //
 // k_render_ellip (render_ellip.cu) evaluates every stamp's K^2 pixel integrals: 253 warp-
 // instructions a stamp at K = 13.  Here a stamp adds its 66 moments to its run's, and a warp turns
-// the runs of a wavelength sample into pixels together: some 75 warp-instructions a stamp at 128 slit
+// the runs of a wavelength sample into pixels together: 79 warp-instructions a stamp at 128 slit
 // points of 8 px (a dozen stamps per run).
 //
 // One CTA of 12 warps takes the items of one slice between two nodes: their four node tables become

@@ -17,8 +17,8 @@
 //
 // Measured on the benchmark's 9216^2 frame of 340 slices x 6000 x 64 stamps: 3.76 ms (the edge tails
 // with their merge 5.2 ms), 4096^2 frame of 40 x 4000 x 32 with its merge 0.24 ms (0.33).  Per stamp
-// 21 warp-instructions; the shared-memory pipe is busy 73 % of the time, the FMA pipe 46 %, issue
-// slots 61 %; four CTAs of 128 threads per SM (128 registers) leave the rest to latency.  Five CTAs
+// 21 warp-instructions; the shared-memory pipe is busy 74 % of the time, the FMA pipe 45 %, issue
+// slots 63 %; four CTAs of 128 threads per SM (128 registers) leave the rest to latency.  Five CTAs
 // spill.  Windows of 9, 13 and 15 px spill at four already (the wide ones hold four pixel pairs'
 // coefficients and a tile quadrant of 7 x 7 pixels) and run three to an SM, with up to 168 registers.
 // It is the faster one at every size: 4096^2 frame of 40 traces x 4000 samples, K = 15, 8 / 32 / 64
