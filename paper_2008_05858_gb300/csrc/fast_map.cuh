@@ -7,7 +7,9 @@
 // 10 packed operations and 4 per axis at degree 5 where the double-float Horner takes 65 packed.
 // The offset's error stays below 6e-7 px (rms 2e-8), so a stamp whose offset is farther than
 // kTieMargin from a pixel edge gets the exact mapping's whole pixel; the few others (one in 1e5),
-// and samples outside the bounds, take the exact mapping itself.
+// and samples outside the bounds, take the exact mapping itself.  Single stamps at the ends of slits bent
+// by the 1 px that s^2 Q may reach: worst pixel 0.74 of the renderer's bound at sigma = 1.0 (0.57 by
+// the exact mapping), rotated PSF 0.98 at 1.3 px (0.69).
 #pragma once
 #include "mixed_common.cuh"
 
